@@ -80,14 +80,11 @@ int sde_mlp_train_step(sde_mlp* net, const float* x, const float* t, uint64_t M,
  * lr_k = lr_final + (lr - lr_final)(1 + cos(pi k / (steps - 1))) / 2; Adam's
  * bias corrections continue the network's step count (earlier
  * sde_mlp_train_step or sde_mlp_fit calls).  losses (device, `steps` floats,
- * or NULL) receives each step's minibatch loss before its update.  One step is
- * captured as a CUDA graph on a private stream and replayed, ordered after
- * the work already on the network's stream; returns when the steps are done.
+ * or NULL) receives each step's minibatch loss before its update.  The steps
+ * (two kernels each) run on a private stream, ordered after the work already
+ * on the network's stream; returns when they are done.
  * Requires 1 <= batch <= min(N, 65536), N <= 2^30, 1 <= steps <= 2^22 (else
- * SDE_EINVAL); the step schedule takes 12 bytes per step on the host and the
- * device for the duration of the call.  No other call may use the same
- * network meanwhile (the capture runs the network's kernels on the private
- * stream). */
+ * SDE_EINVAL).  No other call may use the same network meanwhile. */
 int sde_mlp_fit(sde_mlp* net, const float* X, const float* T, uint64_t N, uint64_t steps,
                 uint32_t batch, float lr, float lr_final, float beta1, float beta2, float eps,
                 uint64_t seed, float* losses);

@@ -66,7 +66,7 @@ def train_ensemble(X, T, shift, scale, log_mask, seeds=(0, 1), steps=8000, batch
                    concurrent=True):
     """Networks on the same labels, one per seed.  X, T: CUDA float32 [N, 7], [N, 2].
     With `concurrent`, each network trains from its own host thread: sde_mlp_fit
-    replays its step graph on a private stream and the binding releases the
+    runs its steps on a private stream and the binding releases the
     interpreter lock during the call, so the small, latency-bound kernels of
     the networks' steps run side by side.  Each network's arithmetic is its
     own, so the trained parameters do not depend on `concurrent`."""
