@@ -291,6 +291,7 @@ __global__ void guided_flags_kernel(const float* __restrict__ v1, const float* _
 struct sde_mlp {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
+    sde_train::Net train{};          // what does not change between training calls
     cudaStream_t fit_stream = nullptr;     // sde_mlp_fit's steps run here, in order after `stream`
     cudaEvent_t fit_ev = nullptr;
     std::string err;
@@ -309,7 +310,7 @@ struct sde_mlp {
     float* Yp = nullptr;             // [cap][8]
     __nv_bfloat16* dY = nullptr;     // [cap][8]
     __nv_bfloat16* dH[3] = {nullptr, nullptr, nullptr};        // [cap][256]
-    double* loss_part = nullptr;     // [cap / 16] partial losses
+    float* res = nullptr;            // [cap][2] residuals
     double* loss64 = nullptr;
     double* host_loss = nullptr;
     int use_tc = 1;                  // forward pass on the fused tcgen05 kernels
@@ -335,8 +336,8 @@ static void free_acts(sde_mlp* n)
         cudaFree(n->A[i]); cudaFree(n->dH[i]);
         n->A[i] = nullptr; n->dH[i] = nullptr;
     }
-    cudaFree(n->Yp); cudaFree(n->dY); cudaFree(n->loss_part);
-    n->Yp = nullptr; n->dY = nullptr; n->loss_part = nullptr;
+    cudaFree(n->Yp); cudaFree(n->dY); cudaFree(n->res);
+    n->Yp = nullptr; n->dY = nullptr; n->res = nullptr;
     n->cap = 0;
 }
 
@@ -356,7 +357,7 @@ static int ensure_acts(sde_mlp* n, uint64_t Mp, bool train)
     MLP_CUDA(n, cudaMalloc(&n->Yp, c * kOutPad * sizeof(float)));
     if (train) {
         MLP_CUDA(n, cudaMalloc(&n->dY, c * kOutPad * sizeof(__nv_bfloat16)));
-        MLP_CUDA(n, cudaMalloc(&n->loss_part, c / 16 * sizeof(double)));
+        MLP_CUDA(n, cudaMalloc(&n->res, c * kOut * sizeof(float)));
     }
     n->cap = c;
     return SDE_OK;
@@ -391,9 +392,9 @@ static cudaError_t forward_rows(sde_mlp* n, uint64_t Mp)
 // The network and its training workspace as the training kernels take them.
 static sde_train::Net train_net(const sde_mlp* n)
 {
-    sde_train::Net t{};
+    sde_train::Net t = n->train;
     t.w = n->w; t.wb = n->wb; t.m1 = n->m1; t.m2 = n->m2; t.maps = n->maps; t.log_mask = n->log_mask;
-    t.X = n->X; t.dY = n->dY; t.loss_part = n->loss_part;
+    t.X = n->X; t.dY = n->dY; t.res = n->res;
     for (int i = 0; i < 3; ++i) { t.A[i] = n->A[i]; t.dH[i] = n->dH[i]; }
     return t;
 }
@@ -437,6 +438,11 @@ int sde_mlp_create(sde_mlp** out, uint64_t seed, void* cuda_stream)
     if (e == cudaSuccess) e = cudaMalloc(&n->loss64, sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&n->tc_error, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(n->tc_error, 0, sizeof(int));
+    if (e == cudaSuccess) e = cudaMalloc(&n->train.loss_part, sde_train::kLossBlocks * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc(&n->train.loss_done, sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaMemset(n->train.loss_done, 0, sizeof(uint32_t));
+    if (e == cudaSuccess) e = sde_train::weight_maps(n->wb, &n->train.w2, &n->train.w3);
+    n->train.error = n->tc_error;
     if (e == cudaSuccess) {
         int dev = 0;
         e = cudaGetDevice(&dev);
@@ -617,6 +623,7 @@ int sde_mlp_fit(sde_mlp* n, const float* X, const float* T, uint64_t N, uint64_t
         const float lr_k = (float)((double)lr_final + 0.5 * ((double)lr - (double)lr_final) * (1.0 + std::cos(pi * frac)));
         b.pos0 = (uint32_t)(k % per_epoch) * batch;
         b.epoch = k / per_epoch;
+        b.settled = k > 0;
         e = sde_train::step(net, b, adam_update(lr_k, beta1, beta2, eps, n->step + k + 1, losses ? losses + k : nullptr),
                             n->fit_stream);
     }
@@ -688,6 +695,7 @@ void sde_mlp_destroy(sde_mlp* n)
     free_acts(n);
     cudaFree(n->w); cudaFree(n->wb); cudaFree(n->grad); cudaFree(n->m1); cudaFree(n->m2);
     cudaFree(n->maps); cudaFree(n->loss64); cudaFree(n->tc_error);
+    cudaFree(n->train.loss_part); cudaFree(n->train.loss_done);
     if (n->host_loss) cudaFreeHost(n->host_loss);
     if (n->fit_stream) cudaStreamDestroy(n->fit_stream);
     if (n->fit_ev) cudaEventDestroy(n->fit_ev);

@@ -3,6 +3,7 @@
 #include <cstddef>
 #include <cstdint>
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -26,11 +27,16 @@ struct Batch {
     uint32_t M;
     uint32_t N, pos0, bits;      // labels, first position, Feistel width (shuffled minibatches)
     unsigned long long seed, epoch;
+    uint32_t settled;            // x, t and the maps were complete before the kernel before this step's began
 };
+
+// Loss sums: blocks of 256 rows, at most 65536 rows.
+constexpr int kLossBlocks = 256;
 
 // The network's parameters and the training workspace for up to cap rows
 // (cap a multiple of 64).
 struct Net {
+    CUtensorMap w2, w3;          // the BF16 copies of W2 and W3 as column blocks of 64 (weight_maps)
     float* w;                    // FP32 master parameters
     __nv_bfloat16* wb;           // BF16 copies
     float* m1;                   // Adam moments
@@ -41,7 +47,10 @@ struct Net {
     __nv_bfloat16* A[3];         // [cap][256] activations
     __nv_bfloat16* dH[3];        // [cap][256] gradients of the pre-activations
     __nv_bfloat16* dY;           // [cap][8] gradient of the standardised outputs
-    double* loss_part;           // [cap / 16] partial losses
+    float* res;                  // [cap][2] residuals y' - t'
+    double* loss_part;           // [kLossBlocks] partial losses
+    uint32_t* loss_done;         // blocks that have written theirs (0 between steps)
+    int* error;                  // set when a wait for a copy ran out
 };
 
 // What to do with the gradients: write them (grad != NULL) or take one Adam
@@ -52,6 +61,9 @@ struct Update {
     float* loss;                 // the batch loss (may be NULL)
     double* loss64;              // the same in FP64 (may be NULL)
 };
+
+// Tensor maps of the BF16 parameter copies wb, for Net.w2 and Net.w3.
+cudaError_t weight_maps(const __nv_bfloat16* wb, CUtensorMap* w2, CUtensorMap* w3);
 
 // Loss and gradients of the batch, then the update; two kernels on `st`.
 cudaError_t step(const Net& n, const Batch& b, const Update& u, cudaStream_t st);
