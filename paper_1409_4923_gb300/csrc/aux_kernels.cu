@@ -17,6 +17,11 @@ cudaError_t launch_segment_m##M(bool, int, int, const PointConsts&, const Launch
                                 const PathOutPtrs&, int, int, int, cudaStream_t);
 SDE_SEG_DECL(0) SDE_SEG_DECL(1) SDE_SEG_DECL(2)
 #undef SDE_SEG_DECL
+#define SDE_SPLIT_DECL(M) \
+cudaError_t launch_split_m##M(bool, int, int, const PointConsts&, const LaunchConsts&, const StatePlanes&, uint32_t, \
+                              uint32_t, const Workspace&, const PathOutPtrs&, cudaStream_t);
+SDE_SPLIT_DECL(0) SDE_SPLIT_DECL(1) SDE_SPLIT_DECL(2)
+#undef SDE_SPLIT_DECL
 #define SDE_CHI_DECL(M) \
 cudaError_t launch_chi_m##M(bool, int, int, const PointConsts&, const LaunchConsts&, uint32_t, \
                             const Workspace&, int, int, int, cudaStream_t);
@@ -59,6 +64,18 @@ cudaError_t launch_segment(int model, bool pois, int dich, int gauss, const Poin
     case kModelOverdampedWashboard:
         return launch_segment_m1(pois, dich, gauss, P, K, M, na, nb, ws, po, bt, gb, sm, st);
     case kModelPWL: return launch_segment_m2(pois, dich, gauss, P, K, M, na, nb, ws, po, bt, gb, sm, st);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+cudaError_t launch_split(int model, bool pois, int dich, int gauss, const PointConsts& P, const LaunchConsts& K,
+                         const StatePlanes& M, uint32_t na, uint32_t nb, const Workspace& ws, const PathOutPtrs& po,
+                         cudaStream_t st)
+{
+    switch (model) {
+    case kModelInertial: return launch_split_m0(pois, dich, gauss, P, K, M, na, nb, ws, po, st);
+    case kModelOverdampedWashboard: return launch_split_m1(pois, dich, gauss, P, K, M, na, nb, ws, po, st);
+    case kModelPWL: return launch_split_m2(pois, dich, gauss, P, K, M, na, nb, ws, po, st);
     default: return cudaErrorInvalidValue;
     }
 }

@@ -460,6 +460,41 @@ int sde_occupancy(sde_ctx* c, int block_threads, int* blocks_per_sm, int* sm_cou
     return SDE_OK;
 }
 
+// Whether coordinates stay below 2^20 between two folds, so that the folds may
+// round by adding 1.5 2^23 (fold<MODEL, true>).  Each step's terms are bounded
+// by the constants: the Gaussian increment by 6 xi (Box-Muller: sqrt(48 ln 2)),
+// a kick by 24 ln 2 zeta; for damping gamma dt <= 1/2 the velocity stays below
+// its initial value plus 8 / (gamma dt) times their sum.
+static bool near_folds(sde_model model, const PointConsts& P)
+{
+    const double step = std::fabs((double)P.fdt) + std::fabs((double)P.a_dt) + std::fabs((double)P.F_dt) +
+                        6.0 * std::fabs((double)P.xi_c) + 24.0 * std::fabs((double)P.zeta_l2) +
+                        std::fabs((double)P.aP_dt) + std::fabs((double)P.Fb_dt) + std::fabs((double)P.mFa_dt);
+    double reach = 4.0 + 4.0 * step;
+    if (model == SDE_INERTIAL_WASHBOARD) {
+        if (!(P.gdt > 0.0f && P.gdt <= 0.5f)) return false;
+        const double v = std::fabs((double)P.v0_lo) + std::fabs((double)P.v0_span) + 8.0 * step / (double)P.gdt;
+        reach = 4.0 + 4.0 * (double)P.wdt * (v + 4.0 * step);
+    }
+    return reach < 1048576.0;      // false for NaN
+}
+
+// Runs of few paths draw their noise in warps of their own (split_kernels.cuh),
+// up to eight 32-path blocks per SM (two integrating warps per scheduler), with
+// Box-Muller up to 24.  Measured (4096 steps, this against one warp per 32 paths
+// with the draws in line, microseconds):
+//   32-path blocks          32          608         1216        1824        3648
+//   Poisson + 3-point    183 / 269   221 / 281   330 / 330   471 / 417   862 / 760
+//   dichotomous + 3-p.   194 / 318   230 / 330   341 / 380   479 / 466   874 / 837
+//   Poisson + Box-M.     218 / 544   292 / 557   454 / 641   686 / 753  1186 / 1331
+//   piecewise-linear P.  281 / 452   296 / 465   391 / 491   590 / 529  1007 / 803
+// A grid set by hand keeps the persistent kernel.
+static bool use_split(const sde_ctx* c, uint64_t items, int dich, int gauss, uint32_t flags, const PointConsts& P)
+{
+    return c->grid_blocks == 0 && items <= (gauss == kGaussNormal ? 24ull : 8ull) * (uint64_t)c->sm_count &&
+           ((flags & SDE_NOISE_POISSON) || dich || gauss) && near_folds(c->model, P);
+}
+
 static int run_impl(sde_ctx* c, uint64_t first_path, uint64_t paths, double dt, uint64_t n_tr,
                     uint64_t n_avg, const sde_path_out* out)
 {
@@ -489,8 +524,13 @@ static int run_impl(sde_ctx* c, uint64_t first_path, uint64_t paths, double dt, 
     const LaunchConsts K = make_launch(c->seed, (uint32_t)items, 0);
     const uint32_t f = c->p.noise_flags;
     const uint64_t total = n_tr + n_avg;
+    const bool split = use_split(c, items, dich_kind(f), gauss_kind(c->p), f, P);
     if (c->steps_per_launch == 0 || c->steps_per_launch >= total) {
-        SDE_CUDA(c, launch_point((int)c->model, (f & SDE_NOISE_POISSON) != 0, dich_kind(f),
+        if (split)
+            SDE_CUDA(c, launch_split((int)c->model, (f & SDE_NOISE_POISSON) != 0, dich_kind(f), gauss_kind(c->p), P, K,
+                                     StatePlanes{nullptr, 0u}, 0u, (uint32_t)total, ws, po, c->stream));
+        else
+            SDE_CUDA(c, launch_point((int)c->model, (f & SDE_NOISE_POISSON) != 0, dich_kind(f),
                                  gauss_kind(c->p), c->paths_per_thread, P, K, ws, po, c->block_threads,
                                  c->grid_blocks, c->sm_count, c->stream));
     } else {
@@ -511,6 +551,11 @@ static int run_impl(sde_ctx* c, uint64_t first_path, uint64_t paths, double dt, 
         const StatePlanes M{(unsigned char*)c->run_state, (uint32_t)(items * 32ull)};
         for (uint64_t na = 0; na < total; na += c->steps_per_launch) {
             const uint64_t nb = std::min(total, na + c->steps_per_launch);
+            if (split) {
+                SDE_CUDA(c, launch_split((int)c->model, (f & SDE_NOISE_POISSON) != 0, dich_kind(f), gauss_kind(c->p), P,
+                                         K, M, (uint32_t)na, (uint32_t)nb, ws, po, c->stream));
+                continue;
+            }
             if (na > 0) SDE_CUDA(c, cudaMemsetAsync(base, 0, 4, c->stream));
             SDE_CUDA(c, launch_segment((int)c->model, (f & SDE_NOISE_POISSON) != 0,
                                        dich_kind(f), gauss_kind(c->p), P, K, M,
@@ -908,9 +953,13 @@ int sde_advance(sde_ctx* c, uint64_t n_steps, const sde_path_out* out, uint64_t*
     const LaunchConsts K = make_launch(r.seed, r.items, 0);
     const StatePlanes M{(unsigned char*)c->state, r.stride};
     const uint32_t f = r.p.noise_flags;
-    SDE_CUDA(c, launch_segment((int)c->model, (f & SDE_NOISE_POISSON) != 0, dich_kind(f),
-                               gauss_kind(r.p), P, K, M, (uint32_t)na, (uint32_t)nb, ws, po,
-                               c->block_threads, c->grid_blocks, c->sm_count, c->stream));
+    if (use_split(c, r.items, dich_kind(f), gauss_kind(r.p), f, P))
+        SDE_CUDA(c, launch_split((int)c->model, (f & SDE_NOISE_POISSON) != 0, dich_kind(f), gauss_kind(r.p), P, K, M,
+                                 (uint32_t)na, (uint32_t)nb, ws, po, c->stream));
+    else
+        SDE_CUDA(c, launch_segment((int)c->model, (f & SDE_NOISE_POISSON) != 0, dich_kind(f),
+                                   gauss_kind(r.p), P, K, M, (uint32_t)na, (uint32_t)nb, ws, po,
+                                   c->block_threads, c->grid_blocks, c->sm_count, c->stream));
     if (last) {
         const uint2 r0 = make_uint2(0u, r.items);
         SDE_CUDA(c, cudaMemcpyAsync(ranges, &r0, sizeof(r0), cudaMemcpyHostToDevice, c->stream));

@@ -160,15 +160,30 @@ struct PathState {
     uint32_t eD, JD, dst, dw1, dw2, dw3;        // dichotomous (Algorithm 4), dst 1 = F_b
 };
 
-template <int MODEL>
+// Whole numbers by adding and subtracting 1.5 2^23, where one unit is the
+// spacing of FP32: rintf and floorf exactly for |x| < 2^22, in two FP32
+// additions instead of a conversion on the SFU pipe (whose latency is several
+// times theirs).  NEAR in the templates below: the caller has made sure that
+// coordinates stay in that range (near_folds on the host).
+constexpr float kRoundShift = 12582912.0f;
+__device__ __forceinline__ float near_rint(float x) { return __fadd_rn(__fadd_rn(x, kRoundShift), -kRoundShift); }
+// floor(0.5 t)
+__device__ __forceinline__ float near_floor_half(float t)
+{
+    return __fadd_rn(__fmaf_rd(t, 0.5f, kRoundShift), -kRoundShift);
+}
+
+template <int MODEL, bool NEAR = false>
 __device__ __forceinline__ void fold(PathState& S)
 {
     if (MODEL == kModelPWL) {
-        const float r = floorf((S.c + 1.0f) * 0.5f);     // c -> [-1, 1), period 2
+        const float t = S.c + 1.0f;
+        const float r = NEAR ? near_floor_half(t) : floorf(t * 0.5f);     // c -> [-1, 1), period 2
         S.c = fmaf(-2.0f, r, S.c);
         S.kf += r;
     } else {
-        const float r = rintf(S.c * 0.15915494309189535f); // c -> [-pi, pi]
+        const float t = __fmul_rn(S.c, 0.15915494309189535f);
+        const float r = NEAR ? near_rint(t) : rintf(t); // c -> [-pi, pi]
         S.c = fmaf(-6.2831853071795865f, r, S.c);
         S.kf += r;
     }
@@ -184,12 +199,13 @@ template <int MODEL> struct FoldPerStep { static constexpr bool value = MODEL !=
 // where no fusion is wanted), so that the compiler's contraction choices
 // cannot differ between the kernels that share this code (one or two paths
 // per lane, segments, scans) and their results stay bit-identical.
-template <int MODEL>
+template <int MODEL, bool NEAR = false>
 __device__ __forceinline__ float add_force_dt(float base, float c, const PointConsts& P)
 {
     if (MODEL == kModelPWL) {
         // V' = +1 on [-1, 0), -1 on [0, 1) (mod 2): force -V0 V'
-        const float y = fmaf(-2.0f, floorf(__fmul_rn(c + 1.0f, 0.5f)), c);
+        const float t = c + 1.0f;
+        const float y = fmaf(-2.0f, NEAR ? near_floor_half(t) : floorf(__fmul_rn(t, 0.5f)), c);
         return base + (y < 0.0f ? -P.fdt : P.fdt);
     } else {
         return fmaf(-P.fdt, cos_sfu(c), base);
@@ -223,7 +239,7 @@ __device__ __forceinline__ float with_jumps(float h1, float pj, float dg)
 // predictor minus the corrector without the jump increments: chi[0] in the
 // coordinate (whdt (v_Euler - v_predictor) = whdt (b1 - b2) / 2 inertial,
 // (b2 - b3) / 2 overdamped), chi[1] in v ((b2 - b3) / 2, inertial).
-template <int MODEL, bool POIS, int DICH, bool ACC, bool FOLD, bool CHI = false>
+template <int MODEL, bool POIS, int DICH, bool ACC, bool FOLD, bool CHI = false, bool NEAR = false>
 __device__ __forceinline__ void pc_step(PathState& S, const PointConsts& P, float dxi, float pj,
                                         float dg, float d0, float d1, float* chi = nullptr)
 {
@@ -232,16 +248,16 @@ __device__ __forceinline__ void pc_step(PathState& S, const PointConsts& P, floa
         d1 += dg;
     }
     if (MODEL == kModelInertial) {
-        const float b1 = add_force_dt<MODEL>(fmaf(-P.gdt, S.v, d0), S.c, P);   // F1_v dt
+        const float b1 = add_force_dt<MODEL, NEAR>(fmaf(-P.gdt, S.v, d0), S.c, P);   // F1_v dt
         const float vxi = S.v + dxi;
         float cb = fmaf(P.wdt, S.v, S.c);                                   // Euler x
         float vb = vxi + b1;                                                // Euler v
-        const float b2 = add_force_dt<MODEL>(fmaf(-P.gdt, vb, d1), cb, P);
+        const float b2 = add_force_dt<MODEL, NEAR>(fmaf(-P.gdt, vb, d1), cb, P);
         const float ch = fmaf(P.whdt, S.v, S.c);
         const float h1 = fmaf(0.5f, b1, vxi);
         cb = fmaf(P.whdt, vb, ch);                                          // predictor x
         vb = fmaf(0.5f, b2, h1);                                            // predictor v
-        const float b3 = add_force_dt<MODEL>(fmaf(-P.gdt, vb, d1), cb, P);
+        const float b3 = add_force_dt<MODEL, NEAR>(fmaf(-P.gdt, vb, d1), cb, P);
         S.c = fmaf(P.whdt, vb, ch);                                         // corrector x
         S.v = fmaf(0.5f, b3, with_jumps<POIS, DICH>(h1, pj, dg));           // corrector v
         accumulate<ACC>(S);
@@ -250,20 +266,20 @@ __device__ __forceinline__ void pc_step(PathState& S, const PointConsts& P, floa
             chi[1] = __fmul_rn(0.5f, b2 - b3);
         }
     } else {
-        const float b1 = add_force_dt<MODEL>(d0, S.c, P);
+        const float b1 = add_force_dt<MODEL, NEAR>(d0, S.c, P);
         const float cxi = S.c + dxi;
         float cb = cxi + b1;                                                // Euler
-        const float b2 = add_force_dt<MODEL>(d1, cb, P);
+        const float b2 = add_force_dt<MODEL, NEAR>(d1, cb, P);
         const float h1 = fmaf(0.5f, b1, cxi);
         cb = fmaf(0.5f, b2, h1);                                            // predictor
-        const float b3 = add_force_dt<MODEL>(d1, cb, P);
+        const float b3 = add_force_dt<MODEL, NEAR>(d1, cb, P);
         S.c = fmaf(0.5f, b3, with_jumps<POIS, DICH>(h1, pj, dg));           // corrector
         if (CHI) {
             chi[0] = __fmul_rn(0.5f, b2 - b3);
             chi[1] = 0.0f;
         }
     }
-    if (FOLD) fold<MODEL>(S);
+    if (FOLD) fold<MODEL, NEAR>(S);
 }
 
 // Algorithm 3 at event JP (step eP): the step's Poissonian increment z - a dt
@@ -1268,14 +1284,25 @@ __device__ __forceinline__ void load_state(PathState& S, const StatePlanes& M, u
     S.dw1 = M.u(7)[path]; S.dw2 = M.u(8)[path]; S.dw3 = M.u(9)[path];
 }
 
-__device__ __forceinline__ void store_state(const PathState& S, const StatePlanes& M, uint32_t path)
+// The coordinates and window sums, and the event counters, of a path.
+__device__ __forceinline__ void store_motion(const PathState& S, const StatePlanes& M, uint32_t path)
 {
     M.d(0)[path] = S.svd; M.d(1)[path] = S.sv2d;
     M.f(0)[path] = S.c; M.f(1)[path] = S.v; M.f(2)[path] = S.kf;
     M.f(3)[path] = S.c_i; M.f(4)[path] = S.kf_i; M.f(5)[path] = S.sv; M.f(6)[path] = S.sv2;
+}
+
+__device__ __forceinline__ void store_events(const PathState& S, const StatePlanes& M, uint32_t path)
+{
     M.u(0)[path] = S.eP; M.u(1)[path] = S.JP; M.u(2)[path] = S.pw2; M.u(3)[path] = S.pw3;
     M.u(4)[path] = S.eD; M.u(5)[path] = S.JD; M.u(6)[path] = S.dst;
     M.u(7)[path] = S.dw1; M.u(8)[path] = S.dw2; M.u(9)[path] = S.dw3;
+}
+
+__device__ __forceinline__ void store_state(const PathState& S, const StatePlanes& M, uint32_t path)
+{
+    store_motion(S, M, path);
+    store_events(S, M, path);
 }
 
 // ---------------------------------------------------------------- reductions

@@ -38,6 +38,14 @@ cudaError_t launch_segment(int model, bool pois, int dich, int gauss, const Poin
                            const Workspace& ws, const PathOutPtrs& po, int block_threads,
                            int grid_blocks, int sm_count, cudaStream_t st);
 
+// Steps [na, nb) of a run or segment (M.base == NULL: a whole run) of few
+// paths, the noise of each 32 paths drawn by warps of its own (split_kernels.cuh);
+// the results are those of
+// launch_point and launch_segment.
+cudaError_t launch_split(int model, bool pois, int dich, int gauss, const PointConsts& P, const LaunchConsts& K,
+                         const StatePlanes& M, uint32_t na, uint32_t nb, const Workspace& ws, const PathOutPtrs& po,
+                         cudaStream_t st);
+
 // Sec. 4's local-error indicator over steps [0, n_steps) of every path:
 // item partials {paths, sum chi_x^2, sum chi_v^2, max |chi_x|, max |chi_v|}.
 cudaError_t launch_chi(int model, bool pois, int dich, int gauss, const PointConsts& P,
