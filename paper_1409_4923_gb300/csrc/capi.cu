@@ -115,9 +115,9 @@ struct sde_ctx {
     uint64_t steps_per_launch = 0;   // 0 = a whole run per launch
     void* run_state = nullptr;    // saved states of runs cut into launches
     size_t run_state_bytes = 0;
-    // scan graphs keyed by (npts, n_items, flags, budget)
+    // scan graphs keyed by (npts, n_items, flags, paths per lane, budget)
     // (and the caller's device output array of sde_scan_device, 0 for sde_scan)
-    std::map<std::tuple<uint32_t, uint32_t, uint32_t, uint64_t, uint64_t>, ScanGraph> graphs;
+    std::map<std::tuple<uint32_t, uint32_t, uint32_t, bool, uint64_t, uint64_t>, ScanGraph> graphs;
     // bumped by every call that writes the workspace; a timed-out scan can be
     // resumed only while its workspace is untouched
     uint64_t ws_gen = 0;
@@ -479,6 +479,13 @@ static bool near_folds(sde_model model, const PointConsts& P)
     return reach < 1048576.0;      // false for NaN
 }
 
+// Paths per lane of a run: the packed pairs of the inertial model fold as
+// near_folds allows, others keep one path per lane (the results are the same).
+static int lane_paths(const sde_ctx* c, bool near)
+{
+    return c->model == SDE_INERTIAL_WASHBOARD && !near ? 1 : c->paths_per_thread;
+}
+
 // Runs of few paths draw their noise in warps of their own (split_kernels.cuh),
 // up to eight 32-path blocks per SM (two integrating warps per scheduler), with
 // Box-Muller up to 24.  Measured (4096 steps, this against one warp per 32 paths
@@ -531,7 +538,7 @@ static int run_impl(sde_ctx* c, uint64_t first_path, uint64_t paths, double dt, 
                                      StatePlanes{nullptr, 0u}, 0u, (uint32_t)total, ws, po, c->stream));
         else
             SDE_CUDA(c, launch_point((int)c->model, (f & SDE_NOISE_POISSON) != 0, dich_kind(f),
-                                 gauss_kind(c->p), c->paths_per_thread, P, K, ws, po, c->block_threads,
+                                 gauss_kind(c->p), lane_paths(c, near_folds(c->model, P)), P, K, ws, po, c->block_threads,
                                  c->grid_blocks, c->sm_count, c->stream));
     } else {
         // Algorithm 5 with `samples` = steps_per_launch: the path states stay
@@ -689,15 +696,22 @@ static int scan_impl(sde_ctx* c, const sde_scan_point* pts, uint32_t npts, sde_s
     const bool use_scan_kernel =
         inertial_scan && (c->scan_mode == 1 ||
                           (c->scan_mode == 0 && (budget > 0 || sum_paths < kPointScanMinPaths * npts)));
-    // Per-point launches of the inertial model take two paths per lane, with
-    // Poisson noise too (measured on the 64 x 64 Poisson scan: 3.75 s against
-    // 3.81 s with one path per lane).
-    const int point_ppt = inertial_scan ? 2 : c->paths_per_thread;
-    // Without Poisson noise the scan kernel takes two paths per lane: a work
-    // item is 64 paths of one point and writes the partial records of its two
-    // 32-path tiles, so each point's records start at an even index (a point
+    // Per-point launches of the inertial model take two paths per lane where
+    // the packed pairs apply (near_folds for every point), with Poisson noise
+    // too (measured on the 64 x 64 Poisson scan: 3.75 s against 3.81 s with one
+    // path per lane).  Without Poisson noise the scan kernel does as well: a
+    // work item is 64 paths of one point and writes the partial records of its
+    // two 32-path tiles, so each point's records start at an even index (a point
     // with an odd tile count leaves one record unused and unfolded).
-    const bool x2 = use_scan_kernel && !(flags & SDE_NOISE_POISSON);
+    bool near = true;
+    for (uint32_t i = 0; i < npts; ++i) {
+        int rc = make_point(c, c->model, pts[i].p, pts[i].dt, pts[i].paths, pts[i].n_transient,
+                            pts[i].n_avg, P[i]);
+        if (rc) return rc;
+        near = near && near_folds(c->model, P[i]);
+    }
+    const int point_ppt = inertial_scan ? (near ? 2 : 1) : lane_paths(c, near);
+    const bool x2 = use_scan_kernel && near && !(flags & SDE_NOISE_POISSON);
     const uint64_t item_paths = x2 ? 64ull : 32ull;
     std::vector<uint2> ranges(npts), items;
     uint64_t total_items = 0;
@@ -711,9 +725,6 @@ static int scan_impl(sde_ctx* c, const sde_scan_point* pts, uint32_t npts, sde_s
         const uint64_t ni = (pts[i].paths + item_paths - 1) / item_paths;
         for (uint64_t t = 0; t < ni; ++t) items.push_back(make_uint2(i, (uint32_t)(item_paths * t)));
         ranges[i] = make_uint2(first, (uint32_t)((pts[i].paths + 31ull) / 32ull));
-        int rc = make_point(c, c->model, pts[i].p, pts[i].dt, pts[i].paths, pts[i].n_transient,
-                            pts[i].n_avg, P[i]);
-        if (rc) return rc;
     }
     const size_t off_items = align256(sizeof(PointConsts) * npts);
     const size_t off_counters = off_items + align256(sizeof(uint2) * total_items);
@@ -739,7 +750,7 @@ static int scan_impl(sde_ctx* c, const sde_scan_point* pts, uint32_t npts, sde_s
     int32_t* h_status = (int32_t*)(c->host + 5 * npts);
     if (use_scan_kernel) {
         const LaunchConsts K = make_launch(c->seed, (uint32_t)total_items, budget);
-        auto key = std::make_tuple(npts, (uint32_t)total_items, flags, budget, (uint64_t)(uintptr_t)dev_out5);
+        auto key = std::make_tuple(npts, (uint32_t)total_items, flags, x2, budget, (uint64_t)(uintptr_t)dev_out5);
         auto it = c->graphs.find(key);
         if (it == c->graphs.end() || c->stream == nullptr) {
             ScanGraph g;

@@ -16,19 +16,10 @@ __device__ __forceinline__ void point_items(const PointConsts& P, const LaunchCo
     const uint32_t lane = threadIdx.x & 31u;
     const uint64_t t0 = K.budget_ns ? globaltimer_ns() : 0ull;
     uint32_t* win = nullptr;
-    if constexpr (WindowedFlips<MODEL, POIS, DICH, GAUSS, PPT>::value) {
-        extern __shared__ uint32_t sde_point_smem[];
-        win = sde_point_smem + (threadIdx.x >> 5) * kWinWordsPerWarp;
-    }
     constexpr bool kKickWin = PPT == 1 && WindowedKicks<POIS, GAUSS>::value;
-    if constexpr (kKickWin) {
-        extern __shared__ uint32_t sde_point_smem[];
-        win = sde_point_smem + (threadIdx.x >> 5) * kKickWordsPerWarp + lane;
-    }
-    if constexpr (WindowedKicks2<MODEL, POIS, DICH, GAUSS, PPT>::value) {
-        extern __shared__ uint32_t sde_point_smem[];
-        win = sde_point_smem + (threadIdx.x >> 5) * kKick2WordsPerWarp;
-    }
+    extern __shared__ __align__(16) uint32_t sde_point_smem[];
+    if constexpr (kKickWin) win = sde_point_smem + (threadIdx.x >> 5) * kKickWordsPerWarp + lane;
+    else win = sde_point_smem + (threadIdx.x >> 5) * X2Words<MODEL, POIS, DICH, GAUSS, PPT>::value;
     for (;;) {
         const uint32_t item = next_item(counter, status, K, lane, t0, (uint32_t)PPT);
         if (item == 0xffffffffu) break;
@@ -76,6 +67,9 @@ __global__ void __launch_bounds__(128) point_kernel(const __grid_constant__ Poin
 // 573 ms against 583 ms at 96 registers (five blocks), 576 ms at 72 and
 // 592 ms at 64, where the spills reach the step loop; uncapped, 123
 // registers and 16 warps, 599 ms), and with Poisson noise in kick windows.
+// With the tables of X2Aux, on 2^20 dichotomous paths x 20,000 steps: 23.1 ms,
+// against 23.8 with five blocks, 23.7 with seven (flip windows of 24 chunks) and
+// 23.5 with eight (16 chunks).
 template <int MODEL, bool POIS, int DICH, int GAUSS, int PPT>
 __global__ void __launch_bounds__(128, 6) point_kernel_capped(const __grid_constant__ PointConsts P,
                                                               const __grid_constant__ LaunchConsts K,
@@ -95,17 +89,13 @@ constexpr auto point_kernel_for()
     else return point_kernel<MODEL, POIS, DICH, GAUSS, PPT>;
 }
 
-// Dynamic shared memory of a launch: the flip or kick windows of its warps.
+// Dynamic shared memory of a launch: the tables and windows of its warps.
 template <int MODEL, bool POIS, int DICH, int GAUSS, int PPT>
 constexpr size_t point_smem_bytes(int block_threads)
 {
-    if (WindowedFlips<MODEL, POIS, DICH, GAUSS, PPT>::value)
-        return (size_t)(block_threads / 32) * kWinWordsPerWarp * sizeof(uint32_t);
-    if (PPT == 1 && WindowedKicks<POIS, GAUSS>::value)
-        return (size_t)(block_threads / 32) * kKickWordsPerWarp * sizeof(uint32_t);
-    if (WindowedKicks2<MODEL, POIS, DICH, GAUSS, PPT>::value)
-        return (size_t)(block_threads / 32) * kKick2WordsPerWarp * sizeof(uint32_t);
-    return 0u;
+    const size_t words = PPT == 1 ? (WindowedKicks<POIS, GAUSS>::value ? kKickWordsPerWarp : 0u)
+                                  : X2Words<MODEL, POIS, DICH, GAUSS, PPT>::value;
+    return (size_t)(block_threads / 32) * words * sizeof(uint32_t);
 }
 
 template <int MODEL, bool POIS, int DICH, int GAUSS, int PPT>

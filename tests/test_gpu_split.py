@@ -81,3 +81,22 @@ def test_far_coordinates_keep_the_conversions(E):
             eng.close()
         np.testing.assert_array_equal(r[0][0], r[1][0])
         np.testing.assert_array_equal(r[0][1], r[1][1])
+
+
+def test_far_coordinates_with_two_paths_per_lane(E):
+    """The same kicks with two paths per lane asked for, in a run and in a scan of
+    one launch per point: both take one path per lane and agree."""
+    r = []
+    for ppt, mode in ((1, 1), (2, 2)):
+        prm = E.make_params(**dict(_params(0, 3), zeta=1e9))
+        eng = E.Engine(0, prm, seed=9)
+        eng.set_tuning(64, 3)
+        eng.set_paths_per_thread(ppt)
+        eng.set_scan_mode(mode)
+        out = _outputs(100)
+        eng.run(100, 0.01, 10, 200, path_out=out)
+        scan = eng.scan([dict(params=prm, dt=0.01, paths=100, n_transient=10, n_avg=200)])
+        r.append((eng.stats()["sums"], scan[0]["sums"], out["X_f"].cpu().numpy()))
+        eng.close()
+    for a, b in zip(*r):
+        np.testing.assert_array_equal(a, b)
