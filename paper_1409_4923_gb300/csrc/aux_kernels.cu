@@ -19,7 +19,9 @@ SDE_SEG_DECL(0) SDE_SEG_DECL(1) SDE_SEG_DECL(2)
 #undef SDE_SEG_DECL
 #define SDE_SPLIT_DECL(M) \
 cudaError_t launch_split_m##M(bool, int, int, const PointConsts&, const LaunchConsts&, const StatePlanes&, uint32_t, \
-                              uint32_t, const Workspace&, const PathOutPtrs&, cudaStream_t);
+                              uint32_t, const Workspace&, const PathOutPtrs&, cudaStream_t); \
+cudaError_t launch_split_chi_m##M(bool, int, int, const PointConsts&, const LaunchConsts&, uint32_t, const Workspace&, \
+                                  cudaStream_t);
 SDE_SPLIT_DECL(0) SDE_SPLIT_DECL(1) SDE_SPLIT_DECL(2)
 #undef SDE_SPLIT_DECL
 #define SDE_CHI_DECL(M) \
@@ -76,6 +78,17 @@ cudaError_t launch_split(int model, bool pois, int dich, int gauss, const PointC
     case kModelInertial: return launch_split_m0(pois, dich, gauss, P, K, M, na, nb, ws, po, st);
     case kModelOverdampedWashboard: return launch_split_m1(pois, dich, gauss, P, K, M, na, nb, ws, po, st);
     case kModelPWL: return launch_split_m2(pois, dich, gauss, P, K, M, na, nb, ws, po, st);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+cudaError_t launch_split_chi(int model, bool pois, int dich, int gauss, const PointConsts& P, const LaunchConsts& K,
+                             uint32_t n_steps, const Workspace& ws, cudaStream_t st)
+{
+    switch (model) {
+    case kModelInertial: return launch_split_chi_m0(pois, dich, gauss, P, K, n_steps, ws, st);
+    case kModelOverdampedWashboard: return launch_split_chi_m1(pois, dich, gauss, P, K, n_steps, ws, st);
+    case kModelPWL: return launch_split_chi_m2(pois, dich, gauss, P, K, n_steps, ws, st);
     default: return cudaErrorInvalidValue;
     }
 }

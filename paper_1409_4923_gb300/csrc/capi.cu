@@ -1102,11 +1102,16 @@ int sde_local_error(sde_ctx* c, uint64_t paths, double dt, uint64_t n_steps, dou
     ++c->ws_gen;
     char* base = (char*)c->ws;
     Workspace ws{(uint32_t*)base, (int32_t*)(base + 4), (double*)(base + L.off_partials)};
-    SDE_CUDA(c, cudaMemsetAsync(base, 0, 8, c->stream));
     const LaunchConsts K = make_launch(c->seed, (uint32_t)items, 0);
     const uint32_t f = c->p.noise_flags;
-    SDE_CUDA(c, launch_chi((int)c->model, (f & SDE_NOISE_POISSON) != 0, dich_kind(f), gauss_kind(c->p), P, K,
+    if (use_split(c, items, dich_kind(f), gauss_kind(c->p), f, P)) {
+        SDE_CUDA(c, launch_split_chi((int)c->model, (f & SDE_NOISE_POISSON) != 0, dich_kind(f), gauss_kind(c->p), P, K,
+                                     (uint32_t)n_steps, ws, c->stream));
+    } else {
+        SDE_CUDA(c, cudaMemsetAsync(base, 0, 8, c->stream));
+        SDE_CUDA(c, launch_chi((int)c->model, (f & SDE_NOISE_POISSON) != 0, dich_kind(f), gauss_kind(c->p), P, K,
                            (uint32_t)n_steps, ws, c->block_threads, c->grid_blocks, c->sm_count, c->stream));
+    }
     SDE_CUDA(c, cudaMemcpyAsync(c->host, ws.partials, 5 * sizeof(double) * items, cudaMemcpyDeviceToHost,
                                 c->stream));
     SDE_CUDA(c, cudaStreamSynchronize(c->stream));

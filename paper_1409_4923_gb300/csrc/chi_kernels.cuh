@@ -10,12 +10,43 @@ __device__ __forceinline__ float warp_max_nonneg(float x)
     return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(x)));
 }
 
+// Running sums and maxima of a path's chi; the FP32 squares are moved to FP64
+// every 256 steps.
+struct ChiSums {
+    double sx = 0.0, sv = 0.0;
+    float ax = 0.0f, av = 0.0f, mx = 0.0f, mv = 0.0f;
+    __device__ __forceinline__ void add(const float (&chi)[2])
+    {
+        ax = fmaf(chi[0], chi[0], ax);
+        av = fmaf(chi[1], chi[1], av);
+        mx = fmaxf(mx, fabsf(chi[0]));
+        mv = fmaxf(mv, fabsf(chi[1]));
+    }
+    __device__ __forceinline__ void flush()
+    {
+        sx += (double)ax;
+        sv += (double)av;
+        ax = av = 0.0f;
+    }
+    // the item's record {paths, sum chi_x^2, sum chi_v^2, max |chi_x|, max |chi_v|}
+    __device__ __forceinline__ void store(double* partials, uint32_t item, uint32_t lane, bool valid)
+    {
+        flush();
+        const double cnt = warp_sum(valid ? 1.0 : 0.0);
+        const double tx = warp_sum(valid ? sx : 0.0), tv = warp_sum(valid ? sv : 0.0);
+        const float hx = warp_max_nonneg(valid ? mx : 0.0f), hv = warp_max_nonneg(valid ? mv : 0.0f);
+        if (lane == 0u) {
+            double* o = partials + 5ull * item;
+            o[0] = cnt; o[1] = tx; o[2] = tv; o[3] = (double)hx; o[4] = (double)hv;
+        }
+    }
+};
+
 // Sec. 4's chi = predictor - corrector (without the jump increments) over
 // steps [0, n_steps) of every path from its initial state, one step at a
 // time with the engine's own step code.  Each 32-path item writes {paths,
 // sum chi_x^2, sum chi_v^2, max |chi_x|, max |chi_v|} (coordinate units for
-// chi_x); the host folds the items.  The FP32 squares are moved to FP64
-// every 256 steps.
+// chi_x); the host folds the items.  Probes of few paths take split_chi_kernel.
 template <int MODEL, bool POIS, int DICH, int GAUSS>
 __global__ void __launch_bounds__(128) chi_kernel(const __grid_constant__ PointConsts P,
                                                   const __grid_constant__ LaunchConsts K, uint32_t n_steps,
@@ -29,8 +60,7 @@ __global__ void __launch_bounds__(128) chi_kernel(const __grid_constant__ PointC
         const uint32_t path = item * 32u + lane;
         PathState S;
         init_path<MODEL, POIS, DICH>(S, P, K, path);
-        double sx = 0.0, sv = 0.0;
-        float ax = 0.0f, av = 0.0f, mx = 0.0f, mv = 0.0f;
+        ChiSums sums;
         for (uint32_t n = 0; n < n_steps; ++n) {
             const float dxi = gauss_at<GAUSS>(P, K, path, n);
             float pj, dg;
@@ -38,28 +68,10 @@ __global__ void __launch_bounds__(128) chi_kernel(const __grid_constant__ PointC
             float chi[2];
             pc_step<MODEL, POIS, DICH, false, true, true>(S, P, dxi, pj, dg, drive_at(n, P), drive_at(n + 1u, P),
                                                           chi);
-            ax = fmaf(chi[0], chi[0], ax);
-            av = fmaf(chi[1], chi[1], av);
-            mx = fmaxf(mx, fabsf(chi[0]));
-            mv = fmaxf(mv, fabsf(chi[1]));
-            if ((n & 255u) == 255u) {
-                sx += (double)ax;
-                sv += (double)av;
-                ax = av = 0.0f;
-            }
+            sums.add(chi);
+            if ((n & 255u) == 255u) sums.flush();
         }
-        sx += (double)ax;
-        sv += (double)av;
-        const bool valid = path < P.n_paths;
-        const double cnt = warp_sum(valid ? 1.0 : 0.0);
-        sx = warp_sum(valid ? sx : 0.0);
-        sv = warp_sum(valid ? sv : 0.0);
-        mx = warp_max_nonneg(valid ? mx : 0.0f);
-        mv = warp_max_nonneg(valid ? mv : 0.0f);
-        if (lane == 0u) {
-            double* o = partials + 5ull * item;
-            o[0] = cnt; o[1] = sx; o[2] = sv; o[3] = (double)mx; o[4] = (double)mv;
-        }
+        sums.store(partials, item, lane, path < P.n_paths);
     }
 }
 

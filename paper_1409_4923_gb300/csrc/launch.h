@@ -52,6 +52,10 @@ cudaError_t launch_chi(int model, bool pois, int dich, int gauss, const PointCon
                        const LaunchConsts& K, uint32_t n_steps, const Workspace& ws, int block_threads,
                        int grid_blocks, int sm_count, cudaStream_t st);
 
+// The same over few paths (split_kernels.cuh).
+cudaError_t launch_split_chi(int model, bool pois, int dich, int gauss, const PointConsts& P, const LaunchConsts& K,
+                             uint32_t n_steps, const Workspace& ws, cudaStream_t st);
+
 // Inertial-washboard scan kernel over an item table of (point, first path);
 // gauss is 0 (no Gaussian noise) or the three-point law.
 cudaError_t launch_scan(bool pois, int dich, int gauss, const PointConsts* pts_dev,

@@ -100,3 +100,17 @@ def test_far_coordinates_with_two_paths_per_lane(E):
         eng.close()
     for a, b in zip(*r):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("model", [0, 1, 2])
+@pytest.mark.parametrize("flags", FLAGS)
+def test_split_probes_equal_persistent_probes(E, model, flags):
+    """Step-size probes (local_error) of few paths against the one-warp kernel."""
+    for paths, steps in ((33, 1), (70, 45), (64, 288), (32, 600)):
+        r = []
+        for grid in (0, 3):
+            eng = E.Engine(model, E.make_params(**_params(model, flags)), seed=9)
+            eng.set_tuning(64, grid)
+            r.append(eng.local_error(paths, 0.01, steps))
+            eng.close()
+        assert r[0] == r[1], (paths, steps)
