@@ -21,11 +21,12 @@
 #include "sde_mlp.h"
 #include "mlp_train.h"
 
+cudaError_t sde_tc_h2_maps(__nv_bfloat16* h2, uint64_t rows, CUtensorMap* store, CUtensorMap* load);
 cudaError_t sde_tc_forward(int M, const float* x, const float* maps, uint32_t log_mask,
-                           const __nv_bfloat16* W1, const float* b1, const __nv_bfloat16* W2,
-                           const float* b2, const __nv_bfloat16* W3, const float* b3,
-                           const __nv_bfloat16* W4, const float* b4, __nv_bfloat16* h2, float* y,
-                           int* error, int sm_count, cudaStream_t st);
+                           const __nv_bfloat16* W1, const float* b1, const CUtensorMap& w2, const float* b2,
+                           const CUtensorMap& w3, const float* b3, const __nv_bfloat16* W4, const float* b4,
+                           const CUtensorMap& h2_store, const CUtensorMap& h2_load, float* y, int* error,
+                           int sm_count, cudaStream_t st);
 
 namespace {
 
@@ -314,6 +315,9 @@ struct sde_mlp {
     double* loss64 = nullptr;
     double* host_loss = nullptr;
     int use_tc = 1;                  // forward pass on the fused tcgen05 kernels
+    __nv_bfloat16* h2 = nullptr;     // their [h2_rows][256] intermediate, and its tensor maps
+    uint64_t h2_rows = 0;
+    CUtensorMap h2_store{}, h2_load{};
     int sm_count = 0;
     int* tc_error = nullptr;         // device word set by a timed-out tensor-core wait
 };
@@ -360,6 +364,23 @@ static int ensure_acts(sde_mlp* n, uint64_t Mp, bool train)
         MLP_CUDA(n, cudaMalloc(&n->res, c * kOut * sizeof(float)));
     }
     n->cap = c;
+    return SDE_OK;
+}
+
+// The tcgen05 forward's intermediate for M rows (whole 128-row tiles).
+static int ensure_h2(sde_mlp* n, uint64_t M)
+{
+    const uint64_t rows = (M + 127u) & ~(uint64_t)127u;
+    if (rows <= n->h2_rows) return SDE_OK;
+    if (n->h2) {
+        cudaStreamSynchronize(n->stream);
+        cudaFree(n->h2);
+        n->h2 = nullptr;
+        n->h2_rows = 0;
+    }
+    MLP_CUDA(n, cudaMalloc(&n->h2, rows * kH * sizeof(__nv_bfloat16)));
+    MLP_CUDA(n, sde_tc_h2_maps(n->h2, rows, &n->h2_store, &n->h2_load));
+    n->h2_rows = rows;
     return SDE_OK;
 }
 
@@ -537,7 +558,8 @@ int sde_mlp_forward(sde_mlp* n, const float* x, uint64_t M, float* y)
     // the tensor-core layers keep their weights resident per CTA: large chunks
     // amortise the weight loads
     const uint64_t chunk = n->use_tc ? kMaxForwardChunk : kMaxBatch;
-    int rc = ensure_acts(n, pad64(M < chunk ? M : chunk), false);
+    const uint64_t rows = M < chunk ? M : chunk;
+    int rc = n->use_tc ? ensure_h2(n, rows) : ensure_acts(n, pad64(rows), false);
     if (rc) return rc;
     for (uint64_t r0 = 0; r0 < M; r0 += chunk) {
         const uint64_t m = (M - r0) < chunk ? (M - r0) : chunk;
@@ -545,9 +567,8 @@ int sde_mlp_forward(sde_mlp* n, const float* x, uint64_t M, float* y)
         if (n->use_tc) {
             // two fused tcgen05 kernels: maps and layers 1-2, layers 3-4 and the output map
             MLP_CUDA(n, sde_tc_forward((int)m, x + r0 * kIn, n->maps, n->log_mask, n->wb + oW1, n->w + oB1,
-                                       n->wb + oW2, n->w + oB2, n->wb + oW3, n->w + oB3, n->wb + oW4,
-                                       n->w + oB4, n->A[1], y + r0 * kOut, n->tc_error, n->sm_count,
-                                       n->stream));
+                                       n->train.w2, n->w + oB2, n->train.w3, n->w + oB3, n->wb + oW4, n->w + oB4,
+                                       n->h2_store, n->h2_load, y + r0 * kOut, n->tc_error, n->sm_count, n->stream));
             continue;
         }
         input_map_kernel<<<nblk(Mp * kInPad), 256, 0, n->stream>>>(x + r0 * kIn, m, Mp, n->maps, n->log_mask, n->X);
@@ -693,6 +714,7 @@ void sde_mlp_destroy(sde_mlp* n)
     if (!n) return;
     if (n->stream || n->own_stream) cudaStreamSynchronize(n->stream);
     free_acts(n);
+    cudaFree(n->h2);
     cudaFree(n->w); cudaFree(n->wb); cudaFree(n->grad); cudaFree(n->m1); cudaFree(n->m2);
     cudaFree(n->maps); cudaFree(n->loss64); cudaFree(n->tc_error);
     cudaFree(n->train.loss_part); cudaFree(n->train.loss_done);

@@ -12,8 +12,8 @@
 // h2 and writes 8 bytes of outputs, instead of the four layers' 3 KB.
 //
 // Each CTA (one per SM) copies its 256 x 256 layer's weights W (BF16, 128 KB)
-// into shared memory once, in the 128-byte-swizzled K-major layout the tensor
-// core reads.  The A operand of a tile moves through a ring of 16 KB slots,
+// into shared memory once, by four tensor copies in the 128-byte-swizzled
+// K-major layout the tensor core reads.  The A operand of a tile moves through a ring of 16 KB slots,
 // one 64-column K-block per slot, so that the A tile of tile t + 1 is written
 // while the tensor core still reads the last blocks of tile t:
 //
@@ -38,7 +38,7 @@
 // grid before they read h2.  The arithmetic is
 // that of the layer-by-layer path (BF16 weights and activations, FP32
 // accumulation and biases) except for the SiLU, evaluated through tanh (see
-// silu_hb).
+// silu_hb2).
 //
 // Every wait is bounded: if an mbarrier phase does not complete within the
 // iteration limit the kernel records an error word, stops, waits for its
@@ -74,10 +74,7 @@ struct TcArgs {
     uint32_t log_mask;               // inputs mapped through log10
     const __nv_bfloat16* W1;         // layers 1-2: [256][16] BF16
     const float* b1;
-    const __nv_bfloat16* A;          // layers 3-4: activations h2 [M][256] BF16
-    const __nv_bfloat16* W;          // this kernel's 256 x 256 layer: [256 out][256 in] BF16
-    const float* b;
-    __nv_bfloat16* out;              // layers 1-2: activations h2 [M][256] BF16
+    const float* b;                  // this kernel's 256 x 256 layer
     const __nv_bfloat16* W4;         // layers 3-4: [8][256] BF16 (rows 0, 1 used)
     const float* b4;
     float* y;                        // layers 3-4: outputs [M][2] in raw units
@@ -108,12 +105,17 @@ constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kN 
 // the half bias hb = b / 2 held in shared memory, h = fma(acc, 1/2, hb) is
 // one rounding of (acc + b) / 2, which equals the rounded sum halved
 // (halving is exact away from subnormals).
-__device__ __forceinline__ float silu_hb(float acc, float hb)
+// Two neighbouring columns at a time, on packed FP32 pairs (2^20 rows: 0.320 ms
+// instead of 0.333 a forward of the 1024 x 1024 screen; the drains issue a
+// fifth fewer instructions).  Twelve drain warps in layers 1-2 instead of eight
+// measured slower again (0.333).
+__device__ __forceinline__ float2 silu_hb2(float a0, float a1, float2 hb)
 {
-    const float h = fmaf(acc, 0.5f, hb);
-    float t;
-    asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(h));
-    return fmaf(h, t, h);
+    const float2 h = __ffma2_rn(make_float2(a0, a1), make_float2(0.5f, 0.5f), hb);
+    float2 t;
+    asm("tanh.approx.f32 %0, %1;" : "=f"(t.x) : "f"(h.x));
+    asm("tanh.approx.f32 %0, %1;" : "=f"(t.y) : "f"(h.y));
+    return __ffma2_rn(h, t, h);
 }
 
 // Four 8 x 8 BF16 matrices to shared memory: lane l gives the address of row
@@ -129,6 +131,16 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b)
 {
     const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
     return *(const uint32_t*)&h;
+}
+
+__device__ __forceinline__ uint32_t pack_bf16x2(float2 a) { return pack_bf16x2(a.x, a.y); }
+
+// Two values rounded to BF16.
+__device__ __forceinline__ float2 bf16_pair(float2 a)
+{
+    const uint32_t w = pack_bf16x2(a);
+    const __nv_bfloat162 h = *(const __nv_bfloat162*)&w;
+    return make_float2(__low2float(h), __high2float(h));
 }
 
 __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3)
@@ -219,8 +231,22 @@ __device__ __forceinline__ void group_sync(uint32_t id, uint32_t count)
 }
 
 // mbarriers of both kernels: full[slot], empty[slot], accumulator full[b],
-// accumulator empty[b], and the issuer's last commit.
-enum { kBarFull = 0, kBarEmpty = 6, kBarAccFull = 12, kBarAccEmpty = 14, kBarDone = 16 };
+// accumulator empty[b], the issuer's last commit, and the weights.
+enum { kBarFull = 0, kBarEmpty = 6, kBarAccFull = 12, kBarAccEmpty = 14, kBarDone = 16, kBarW = 17 };
+
+// The layer's weights to sB (one thread).  The MMA issuer waits for them; the
+// producers and the drain do not need them.
+__device__ __forceinline__ void load_weights(uint32_t sB, const CUtensorMap& tmW, uint32_t bar0)
+{
+    const uint32_t bar = bar0 + 8u * kBarW;
+    asm volatile("fence.proxy.async;" ::: "memory");      // barriers and weights were written by ordinary stores
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bar), "r"((uint32_t)kBBytes) : "memory");
+    for (uint32_t c = 0; c < (uint32_t)kKBlocks; ++c)
+        asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
+                     " [%0], [%1, {%2, %3}], [%4];"
+                     :: "r"(sB + c * (uint32_t)kBRegion), "l"((uint64_t)&tmW), "r"((int)c * kKBlock), "r"(0), "r"(bar)
+                     : "memory");
+}
 
 constexpr int kL12Threads = 800;      // warps 0-7 drain, 8-23 produce, 24 issues the MMAs
 constexpr int kL12Drain = 256;
@@ -230,7 +256,7 @@ constexpr int kL12OffB = 0;
 constexpr int kL12OffA = kBBytes;
 constexpr int kL12OffStage = kL12OffA + kL12Slots * kARegion;    // 8 drain warps x 2 KB (32 rows x 32 columns)
 constexpr int kL12OffBar = kL12OffStage + (kL12Drain / 32) * 2048;
-constexpr int kL12OffTslot = kL12OffBar + 192;             // after the 17 mbarriers
+constexpr int kL12OffTslot = kL12OffBar + 192;             // after the 18 mbarriers
 constexpr int kL12OffBias = kL12OffBar + 256;
 constexpr int kL12OffX = kL12OffBias + kN * 4;                   // 16 producer warps x 16 x 24 BF16
 constexpr int kL12OffW1 = kL12OffX + 16 * 16 * kXStride * 2;      // 256 x 24 BF16
@@ -252,6 +278,7 @@ static_assert(kL12SmemBytes <= 227 * 1024, "shared memory");
 // memory (one 16-byte store per lane and row would touch 32 cache lines per
 // instruction).
 __global__ void __launch_bounds__(kL12Threads, 1) mlp_tc_layers12_kernel(const __grid_constant__ TcArgs g,
+                                                                       const __grid_constant__ CUtensorMap tmW,
                                                                        const __grid_constant__ CUtensorMap tmH)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -283,17 +310,14 @@ __global__ void __launch_bounds__(kL12Threads, 1) mlp_tc_layers12_kernel(const _
             mbar_init(bar0 + 8u * (kBarAccEmpty + b), (uint32_t)(kL12Drain / 32));
         }
         mbar_init(bar0 + 8u * kBarDone, 1u);
+        mbar_init(bar0 + 8u * kBarW, 1u);
+        load_weights(smem_addr(sB), tmW, bar0);
     }
     for (uint32_t i = tid; i < (uint32_t)kN; i += (uint32_t)kL12Threads) sbias[i] = 0.5f * g.b[i];   // half biases
     if (tid < 18u) smaps[tid] = g.maps[tid];
     for (uint32_t i = tid; i < (uint32_t)kN * 2u; i += (uint32_t)kL12Threads)   // 2 x 16 bytes per row
         *(uint4*)(sW1 + (i >> 1) * kXStride + (i & 1u) * 8u) = *(const uint4*)(g.W1 + (size_t)(i >> 1) * 16u + (i & 1u) * 8u);
     for (uint32_t i = tid; i < (uint32_t)kN; i += (uint32_t)kL12Threads) sb1[i] = 0.5f * g.b1[i];
-    for (uint32_t i = tid; i < (uint32_t)kN * (kK / 8); i += (uint32_t)kL12Threads) {
-        const uint32_t n = i / (kK / 8), c = i % (kK / 8);
-        const uint4 v = *(const uint4*)(g.W + (size_t)n * kK + c * 8u);
-        *(uint4*)(sB + (c >> 3) * kBRegion + sw128(n, c & 7u)) = v;
-    }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -375,8 +399,8 @@ __global__ void __launch_bounds__(kL12Threads, 1) mlp_tc_layers12_kernel(const _
 #pragma unroll
                     for (uint32_t m = 0; m < 4u; ++m) {
                         const uint32_t nt = 2u * pp + (m >> 1), h = m & 1u;
-                        const uint32_t col = kb * 64u + nt * 8u + 2u * ti;
-                        wv[m] = pack_bf16x2(silu_hb(acc[nt][2 * h], sb1[col]), silu_hb(acc[nt][2 * h + 1], sb1[col + 1]));
+                        const float2 hb = *(const float2*)(sb1 + kb * 64u + nt * 8u + 2u * ti);
+                        wv[m] = pack_bf16x2(silu_hb2(acc[nt][2 * h], acc[nt][2 * h + 1], hb));
                     }
                     stsm_x4(sA_a + slot * (uint32_t)kARegion + sw128(srow, 2u * pp + (lane >> 4)), wv[0], wv[1], wv[2], wv[3]);
                 }
@@ -387,6 +411,7 @@ __global__ void __launch_bounds__(kL12Threads, 1) mlp_tc_layers12_kernel(const _
     } else if (warp == 24u) {
         // MMA issuer: block c of tile i once its 256 producer threads have arrived
         if (lane == 0) {
+            ok = wait_phase(bar0 + 8u * kBarW, 0u);
             for (int i = 0; i < ntile && ok; ++i) {
                 const uint32_t b = (uint32_t)i & 1u;
                 if (i >= 2 && !wait_phase(bar0 + 8u * (kBarAccEmpty + b), (uint32_t)((i >> 1) - 1) & 1u)) {
@@ -419,6 +444,7 @@ __global__ void __launch_bounds__(kL12Threads, 1) mlp_tc_layers12_kernel(const _
             }
             mma_commit(bar0 + 8u * kBarDone);
             wait_phase(bar0 + 8u * kBarDone, 0u);
+            wait_phase(bar0 + 8u * kBarW, 0u);      // no copy may still be in flight when the block exits
         }
         __syncwarp();
     } else if (warp < 8u) {
@@ -454,9 +480,13 @@ __global__ void __launch_bounds__(kL12Threads, 1) mlp_tc_layers12_kernel(const _
                 const uint32_t cb = c0 + 16u * j;
                 uint32_t packed[8];
 #pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    packed[k] = pack_bf16x2(silu_hb(__uint_as_float(cur[2 * k]), sbias[cb + 2 * k]),
-                                            silu_hb(__uint_as_float(cur[2 * k + 1]), sbias[cb + 2 * k + 1]));
+                for (int k = 0; k < 4; ++k) {
+                    const float4 hb = *(const float4*)(sbias + cb + 4 * k);
+                    packed[2 * k] = pack_bf16x2(silu_hb2(__uint_as_float(cur[4 * k]), __uint_as_float(cur[4 * k + 1]),
+                                                         make_float2(hb.x, hb.y)));
+                    packed[2 * k + 1] = pack_bf16x2(silu_hb2(__uint_as_float(cur[4 * k + 2]),
+                                                             __uint_as_float(cur[4 * k + 3]), make_float2(hb.z, hb.w)));
+                }
                 if ((j & 1u) == 0u) {
                     // the previous tensor store has read the staging block
                     if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -510,7 +540,7 @@ constexpr int kL34Drain = 512;
 constexpr int kL34Slots = 4;          // one tile's four K-blocks (a fifth slot measured no faster)
 constexpr int kL34OffB = 0;
 constexpr int kL34OffA = kBBytes;
-constexpr int kL34OffBar = kL34OffA + kL34Slots * kARegion;       // 17 mbarriers
+constexpr int kL34OffBar = kL34OffA + kL34Slots * kARegion;       // 18 mbarriers
 constexpr int kL34OffTslot = kL34OffBar + 192;
 constexpr int kL34OffBias = kL34OffBar + 256;
 constexpr int kL34OffW4 = kL34OffBias + kN * 4;
@@ -520,6 +550,7 @@ constexpr int kL34SmemBytes = kL34OffMaps + 64 * 4 + 1024;
 static_assert(kL34SmemBytes <= 227 * 1024, "shared memory");
 
 __global__ void __launch_bounds__(kL34Threads, 1) mlp_tc_layers34_kernel(const __grid_constant__ TcArgs g,
+                                                                      const __grid_constant__ CUtensorMap tmW,
                                                                       const __grid_constant__ CUtensorMap tmA)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -549,16 +580,13 @@ __global__ void __launch_bounds__(kL34Threads, 1) mlp_tc_layers34_kernel(const _
             mbar_init(bar0 + 8u * (kBarAccEmpty + b), (uint32_t)(kL34Drain / 32));
         }
         mbar_init(bar0 + 8u * kBarDone, 1u);
+        mbar_init(bar0 + 8u * kBarW, 1u);
+        load_weights(smem_addr(sB), tmW, bar0);
     }
     for (uint32_t i = tid; i < (uint32_t)kN; i += (uint32_t)kL34Threads) sbias[i] = 0.5f * g.b[i];   // half biases
     if (tid < 18u) smaps[tid] = g.maps[tid];
     for (uint32_t i = tid; i < (uint32_t)(kOut * kN); i += (uint32_t)kL34Threads) sW4[i] = __bfloat162float(g.W4[i]);
     if (tid < (uint32_t)kOut) smaps[32 + tid] = g.b4[tid];
-    for (uint32_t i = tid; i < (uint32_t)kN * (kK / 8); i += (uint32_t)kL34Threads) {
-        const uint32_t n = i / (kK / 8), c = i % (kK / 8);
-        const uint4 v = *(const uint4*)(g.W + (size_t)n * kK + c * 8u);
-        *(uint4*)(sB + (c >> 3) * kBRegion + sw128(n, c & 7u)) = v;
-    }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -601,6 +629,7 @@ __global__ void __launch_bounds__(kL34Threads, 1) mlp_tc_layers34_kernel(const _
     } else if (warp == 17) {
         // MMA issuer: block c of tile i as soon as it has landed
         if (lane == 0) {
+            ok = wait_phase(bar0 + 8u * kBarW, 0u);
             for (int i = 0; i < ntile && ok; ++i) {
                 const uint32_t b = (uint32_t)i & 1u;
                 if (i >= 2 && !wait_phase(bar0 + 8u * (kBarAccEmpty + b), (uint32_t)((i >> 1) - 1) & 1u)) {
@@ -632,6 +661,7 @@ __global__ void __launch_bounds__(kL34Threads, 1) mlp_tc_layers34_kernel(const _
             // every MMA of this thread completes before the tensor memory is released
             mma_commit(bar0 + 8u * kBarDone);
             wait_phase(bar0 + 8u * kBarDone, 0u);
+            wait_phase(bar0 + 8u * kBarW, 0u);      // no copy may still be in flight when the block exits
         }
         __syncwarp();
     } else if (warp < 16u) {
@@ -665,14 +695,16 @@ __global__ void __launch_bounds__(kL34Threads, 1) mlp_tc_layers34_kernel(const _
                              : "r"(taddr + cb));
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const uint32_t w = pack_bf16x2(silu_hb(__uint_as_float(v[2 * j]), sbias[cb + 2 * j]),
-                                                   silu_hb(__uint_as_float(v[2 * j + 1]), sbias[cb + 2 * j + 1]));
-                    const __nv_bfloat162 h = *(const __nv_bfloat162*)&w;
-                    const float h0 = __low2float(h), h1 = __high2float(h);
-                    const uint32_t c = cb + 2u * (uint32_t)j;
-                    p0 = fmaf(h1, sW4[c + 1], fmaf(h0, sW4[c], p0));
-                    p1 = fmaf(h1, sW4[kN + c + 1], fmaf(h0, sW4[kN + c], p1));
+                for (uint32_t k = 0; k < 8u; ++k) {
+                    const uint32_t c = cb + 4u * k;
+                    const float4 hb = *(const float4*)(sbias + c), w0 = *(const float4*)(sW4 + c),
+                                 w1 = *(const float4*)(sW4 + kN + c);
+                    const float2 ha = bf16_pair(silu_hb2(__uint_as_float(v[4 * k]), __uint_as_float(v[4 * k + 1]),
+                                                         make_float2(hb.x, hb.y)));
+                    const float2 hc = bf16_pair(silu_hb2(__uint_as_float(v[4 * k + 2]), __uint_as_float(v[4 * k + 3]),
+                                                         make_float2(hb.z, hb.w)));
+                    p0 = fmaf(hc.y, w0.w, fmaf(hc.x, w0.z, fmaf(ha.y, w0.y, fmaf(ha.x, w0.x, p0))));
+                    p1 = fmaf(hc.y, w1.w, fmaf(hc.x, w1.z, fmaf(ha.y, w1.y, fmaf(ha.x, w1.x, p1))));
                 }
             }
             // this warp is done with the accumulator half
@@ -728,26 +760,37 @@ static EncodeTiledFn lookup_encode_tiled()
     return (EncodeTiledFn)p;
 }
 
-// Layers 3-4 over h2 [M][256] (BF16): the tensor map describes h2 as a
-// 2-D tensor of M rows and 256 columns whose 128-row x 64-column boxes land
-// in the 128-byte-swizzled K-major layout of the tensor core's A operand.
-static cudaError_t launch_layers34(const sde_tc::TcArgs& a, int sm_count, cudaStream_t st)
+// Tensor maps of the activations h2 [rows][256] (BF16) for the forward's two
+// kernels: layers 1-2 store 32 x 32 boxes from 64-byte-swizzled staging blocks,
+// layers 3-4 load 128-row x 64-column boxes in the 128-byte-swizzled K-major
+// layout of the tensor core's A operand.  They describe the whole buffer, so
+// they serve every call: rows past the call's M that its last tile covers are
+// stored and loaded like the others, and their outputs are not written.
+cudaError_t sde_tc_h2_maps(__nv_bfloat16* h2, uint64_t rows, CUtensorMap* store, CUtensorMap* load)
 {
     static const EncodeTiledFn encode = lookup_encode_tiled();
     if (!encode) return cudaErrorNotSupported;
+    const cuuint64_t dims[2] = {(cuuint64_t)sde_tc::kK, (cuuint64_t)rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)sde_tc::kK * sizeof(__nv_bfloat16)};
+    const cuuint32_t sbox[2] = {32u, 32u}, lbox[2] = {(cuuint32_t)sde_tc::kKBlock, (cuuint32_t)sde_tc::kRows};
+    const cuuint32_t estr[2] = {1u, 1u};
+    if (encode(store, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void*)h2, dims, strides, sbox, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS ||
+        encode(load, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void*)h2, dims, strides, lbox, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+    return cudaSuccess;
+}
+
+static cudaError_t launch_layers34(const sde_tc::TcArgs& a, const CUtensorMap& w3, const CUtensorMap& h2_load,
+                                   int sm_count, cudaStream_t st)
+{
     // the attribute belongs to the current device: set it on every launch
     cudaError_t e = cudaFuncSetAttribute(sde_tc::mlp_tc_layers34_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          sde_tc::kL34SmemBytes);
     if (e != cudaSuccess) return e;
-    alignas(64) CUtensorMap tm;
-    const cuuint64_t dims[2] = {(cuuint64_t)sde_tc::kK, (cuuint64_t)a.M};
-    const cuuint64_t strides[1] = {(cuuint64_t)sde_tc::kK * sizeof(__nv_bfloat16)};
-    const cuuint32_t box[2] = {(cuuint32_t)sde_tc::kKBlock, (cuuint32_t)sde_tc::kRows};
-    const cuuint32_t estr[2] = {1u, 1u};
-    if (encode(&tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void*)a.A, dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorInvalidValue;
     const int tiles = (a.M + sde_tc::kRows - 1) / sde_tc::kRows;
     const int grid = tiles < sm_count ? tiles : sm_count;
     // programmatic dependent launch: the kernel waits for the layers 1-2 grid
@@ -762,50 +805,39 @@ static cudaError_t launch_layers34(const sde_tc::TcArgs& a, int sm_count, cudaSt
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, sde_tc::mlp_tc_layers34_kernel, a, tm);
+    return cudaLaunchKernelEx(&cfg, sde_tc::mlp_tc_layers34_kernel, a, w3, h2_load);
 }
 
-static cudaError_t launch_layers12(const sde_tc::TcArgs& a, int sm_count, cudaStream_t st)
+static cudaError_t launch_layers12(const sde_tc::TcArgs& a, const CUtensorMap& w2, const CUtensorMap& h2_store,
+                                   int sm_count, cudaStream_t st)
 {
-    static const EncodeTiledFn encode = lookup_encode_tiled();
-    if (!encode) return cudaErrorNotSupported;
     // the attribute belongs to the current device: set it on every launch
     cudaError_t e = cudaFuncSetAttribute(sde_tc::mlp_tc_layers12_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          sde_tc::kL12SmemBytes);
     if (e != cudaSuccess) return e;
-    // h2 [M][256] BF16 written in 32 x 32 boxes from 64-byte-swizzled staging blocks
-    alignas(64) CUtensorMap tm;
-    const cuuint64_t dims[2] = {(cuuint64_t)sde_tc::kN, (cuuint64_t)a.M};
-    const cuuint64_t strides[1] = {(cuuint64_t)sde_tc::kN * sizeof(__nv_bfloat16)};
-    const cuuint32_t box[2] = {32u, 32u};
-    const cuuint32_t estr[2] = {1u, 1u};
-    if (encode(&tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void*)a.out, dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorInvalidValue;
     const int tiles = (a.M + sde_tc::kRows - 1) / sde_tc::kRows;
     const int grid = tiles < sm_count ? tiles : sm_count;
-    sde_tc::mlp_tc_layers12_kernel<<<grid, sde_tc::kL12Threads, sde_tc::kL12SmemBytes, st>>>(a, tm);
+    sde_tc::mlp_tc_layers12_kernel<<<grid, sde_tc::kL12Threads, sde_tc::kL12SmemBytes, st>>>(a, w2, h2_store);
     return cudaGetLastError();
 }
 
 // Host launcher (used by mlp.cu): the forward pass of M rows of raw inputs x
-// [M][7] to raw outputs y [M][2], with h2 [M][256] (BF16) as the one
-// intermediate in global memory.  Weight pointers are the BF16 copies of the
-// parameter vector; biases and maps are FP32.
+// [M][7] to raw outputs y [M][2], with h2 (BF16, a multiple of 128 rows) as the
+// one intermediate in global memory.  w2, w3: tensor maps of the layers'
+// weights (sde_train::weight_maps); the other weight pointers are the BF16
+// copies of the parameter vector; biases and maps are FP32.
 cudaError_t sde_tc_forward(int M, const float* x, const float* maps, uint32_t log_mask,
-                           const __nv_bfloat16* W1, const float* b1, const __nv_bfloat16* W2,
-                           const float* b2, const __nv_bfloat16* W3, const float* b3,
-                           const __nv_bfloat16* W4, const float* b4, __nv_bfloat16* h2, float* y,
-                           int* error, int sm_count, cudaStream_t st)
+                           const __nv_bfloat16* W1, const float* b1, const CUtensorMap& w2, const float* b2,
+                           const CUtensorMap& w3, const float* b3, const __nv_bfloat16* W4, const float* b4,
+                           const CUtensorMap& h2_store, const CUtensorMap& h2_load, float* y, int* error,
+                           int sm_count, cudaStream_t st)
 {
     if (M <= 0) return cudaSuccess;
     sde_tc::TcArgs a{};
-    a.M = M; a.x = x; a.maps = maps; a.log_mask = log_mask; a.W1 = W1; a.b1 = b1;
-    a.W = W2; a.b = b2; a.out = h2; a.error = error;
-    cudaError_t e = launch_layers12(a, sm_count, st);
+    a.M = M; a.x = x; a.maps = maps; a.log_mask = log_mask; a.W1 = W1; a.b1 = b1; a.b = b2; a.error = error;
+    cudaError_t e = launch_layers12(a, w2, h2_store, sm_count, st);
     if (e != cudaSuccess) return e;
     sde_tc::TcArgs c{};
-    c.M = M; c.maps = maps; c.A = h2; c.W = W3; c.b = b3; c.W4 = W4; c.b4 = b4; c.y = y; c.error = error;
-    return launch_layers34(c, sm_count, st);
+    c.M = M; c.maps = maps; c.b = b3; c.W4 = W4; c.b4 = b4; c.y = y; c.error = error;
+    return launch_layers34(c, w3, h2_load, sm_count, st);
 }
