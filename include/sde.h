@@ -281,7 +281,10 @@ int sde_philox_words(sde_ctx* ctx, const uint32_t* ctr, uint64_t n, uint64_t see
 
 /* Launch shape of the path kernels of this context: threads per block
  * (32..128, multiple of 32) and blocks in the grid (0 = one persistent wave
- * from the occupancy calculator).  Results never depend on the shape; the
+ * from the occupancy calculator).  Without a grid, runs, segments and step-size
+ * probes of few paths (up to eight 32-path blocks per SM, 24 with Box-Muller
+ * increments) take kernels whose noise is drawn by warps of their own, and the
+ * block size does not apply to them.  Results never depend on the shape; the
  * autotuner of the Python layer picks it.  EINVAL outside those ranges.
  * Tuning aid: the paper fixes no launch shape (Sec. 5 only asks for enough
  * threads per block to keep the GPU busy). */
@@ -292,18 +295,20 @@ int sde_set_tuning(sde_ctx* ctx, int block_threads, int grid_blocks);
  * dependency chains hide each other's latencies and the drive values and
  * loop work are shared; each path takes exactly the operations it takes with
  * 1, so results do not change.  Applies to sde_run, sde_run_paths and the
- * per-point launches of sde_scan for the overdamped models.  EINVAL otherwise.
+ * per-point launches of sde_scan for the overdamped models, and not to runs of
+ * few paths (sde_set_tuning) or to parameters whose kicks throw the particle
+ * past 2^20 in a step.  EINVAL otherwise.
  * Tuning aid with no counterpart in the paper, which runs one path per
  * thread (Algorithm 5). */
 int sde_set_paths_per_thread(sde_ctx* ctx, int paths_per_thread);
 
 /* How sde_scan runs the points of the inertial model: 0 (default) chooses
  * one point-kernel launch per point when the points have 2048 paths or more
- * on average (64 such launches side by side fill the GPU) and no deadline is
+ * on average (128 such launches side by side fill the GPU) and no deadline is
  * given, and the persistent scan kernel otherwise; 1 always the persistent
  * scan kernel; 2 always one launch per point.  With one launch per point a
- * deadline bounds each launch's device time from that launch's own start.  The launches of mode 2 run side by side on side streams of the
- * context, each with its point's constants as kernel arguments.  Results do
+ * deadline bounds each launch's device time from that launch's own start.  The
+ * launches of mode 2 run side by side on side streams of the context, each with its point's constants as kernel arguments.  Results do
  * not depend on the mode.  The other models always run one launch per point.
  * Tuning aid with no counterpart in the paper.  EINVAL outside 0..2. */
 int sde_set_scan_mode(sde_ctx* ctx, int mode);

@@ -93,8 +93,8 @@ int sde_mlp_fit(sde_mlp* net, const float* X, const float* T, uint64_t N, uint64
  * fifth-generation tensor cores (input map and layers 1-2; layers 3-4 and
  * the output map; tcgen05.mma with FP32 accumulators in tensor memory,
  * persistent CTAs holding a 256 x 256 layer's weights in shared memory, SiLU
- * through tanh), 0 the layer-by-layer warp-level mma.sync kernels that also
- * serve training.  Results agree within the BF16 rounding of the
+ * through tanh), 0 the layer-by-layer warp-level mma.sync kernels.  Training
+ * has kernels of its own (mma.sync).  Results agree within the BF16 rounding of the
  * activations. */
 int sde_mlp_set_tensor_path(sde_mlp* net, int use_tcgen05);
 

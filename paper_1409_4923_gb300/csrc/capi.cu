@@ -10,6 +10,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <limits>
 #include <map>
 #include <string>
 #include <tuple>
@@ -57,6 +58,7 @@ struct SegmentedRun {
     uint64_t paths = 0, n_tr = 0, n_avg = 0, n_done = 0;
     double dt = 0.0;
     uint32_t items = 0, stride = 0;
+    double c0 = 0.0, v0 = 0.0;       // largest coordinate and velocity of restored states
 };
 
 // Checkpoint header (host byte order; followed by the saved states).
@@ -464,17 +466,18 @@ int sde_occupancy(sde_ctx* c, int block_threads, int* blocks_per_sm, int* sm_cou
 // round by adding 1.5 2^23 (fold<MODEL, true>).  Each step's terms are bounded
 // by the constants: the Gaussian increment by 6 xi (Box-Muller: sqrt(48 ln 2)),
 // a kick by 24 ln 2 zeta; for damping gamma dt <= 1/2 the velocity stays below
-// its initial value plus 8 / (gamma dt) times their sum.
-static bool near_folds(sde_model model, const PointConsts& P)
+// its initial value plus 8 / (gamma dt) times their sum.  c0, v0: the largest
+// coordinate and velocity of states that come from a checkpoint.
+static bool near_folds(sde_model model, const PointConsts& P, double c0 = 0.0, double v0 = 0.0)
 {
     const double step = std::fabs((double)P.fdt) + std::fabs((double)P.a_dt) + std::fabs((double)P.F_dt) +
                         6.0 * std::fabs((double)P.xi_c) + 24.0 * std::fabs((double)P.zeta_l2) +
                         std::fabs((double)P.aP_dt) + std::fabs((double)P.Fb_dt) + std::fabs((double)P.mFa_dt);
-    double reach = 4.0 + 4.0 * step;
+    double reach = 4.0 + c0 + 4.0 * step;
     if (model == SDE_INERTIAL_WASHBOARD) {
         if (!(P.gdt > 0.0f && P.gdt <= 0.5f)) return false;
-        const double v = std::fabs((double)P.v0_lo) + std::fabs((double)P.v0_span) + 8.0 * step / (double)P.gdt;
-        reach = 4.0 + 4.0 * (double)P.wdt * (v + 4.0 * step);
+        const double v = v0 + std::fabs((double)P.v0_lo) + std::fabs((double)P.v0_span) + 8.0 * step / (double)P.gdt;
+        reach = 4.0 + c0 + 4.0 * (double)P.wdt * (v + 4.0 * step);
     }
     return reach < 1048576.0;      // false for NaN
 }
@@ -496,10 +499,11 @@ static int lane_paths(const sde_ctx* c, bool near)
 //   Poisson + Box-M.     218 / 544   292 / 557   454 / 641   686 / 753  1186 / 1331
 //   piecewise-linear P.  281 / 452   296 / 465   391 / 491   590 / 529  1007 / 803
 // A grid set by hand keeps the persistent kernel.
-static bool use_split(const sde_ctx* c, uint64_t items, int dich, int gauss, uint32_t flags, const PointConsts& P)
+static bool use_split(const sde_ctx* c, uint64_t items, int dich, int gauss, uint32_t flags, const PointConsts& P,
+                      double c0 = 0.0, double v0 = 0.0)
 {
     return c->grid_blocks == 0 && items <= (gauss == kGaussNormal ? 24ull : 8ull) * (uint64_t)c->sm_count &&
-           ((flags & SDE_NOISE_POISSON) || dich || gauss) && near_folds(c->model, P);
+           ((flags & SDE_NOISE_POISSON) || dich || gauss) && near_folds(c->model, P, c0, v0);
 }
 
 static int run_impl(sde_ctx* c, uint64_t first_path, uint64_t paths, double dt, uint64_t n_tr,
@@ -964,7 +968,7 @@ int sde_advance(sde_ctx* c, uint64_t n_steps, const sde_path_out* out, uint64_t*
     const LaunchConsts K = make_launch(r.seed, r.items, 0);
     const StatePlanes M{(unsigned char*)c->state, r.stride};
     const uint32_t f = r.p.noise_flags;
-    if (use_split(c, r.items, dich_kind(f), gauss_kind(r.p), f, P))
+    if (use_split(c, r.items, dich_kind(f), gauss_kind(r.p), f, P, r.c0, r.v0))
         SDE_CUDA(c, launch_split((int)c->model, (f & SDE_NOISE_POISSON) != 0, dich_kind(f), gauss_kind(r.p), P, K, M,
                                  (uint32_t)na, (uint32_t)nb, ws, po, c->stream));
     else
@@ -1071,6 +1075,11 @@ int sde_restore(sde_ctx* c, const void* buf, uint64_t bytes)
             return w;
         };
         for (uint32_t i = 0; i < r.stride; ++i) {
+            float cv[2];             // planes 0 (c) and 1 (v) of the float block
+            for (int k = 0; k < 2; ++k) std::memcpy(cv + k, src + 16ull * r.stride + 4ull * ((uint64_t)k * r.stride + i), 4);
+            const double big = std::numeric_limits<double>::infinity();      // for NaN too: no near folds
+            r.c0 = std::max(r.c0, std::isnan(cv[0]) ? big : std::fabs((double)cv[0]));
+            r.v0 = std::max(r.v0, std::isnan(cv[1]) ? big : std::fabs((double)cv[1]));
             if (pois && (word(0, i) < r.n_done || word(1, i) < 1u))
                 return fail(c, SDE_EINVAL, "checkpoint: invalid Poisson event counter");
             if (dich && (word(4, i) < r.n_done || word(5, i) < 1u || word(6, i) > 1u))

@@ -103,6 +103,36 @@ def test_far_coordinates_with_two_paths_per_lane(E):
 
 
 @pytest.mark.parametrize("model", [0, 1, 2])
+def test_far_coordinates_in_a_checkpoint(E, model):
+    """A checkpoint whose coordinates and velocities lie beyond the near folds'
+    range (its checksum valid): a restored run keeps the conversions."""
+    eng = E.Engine(model, E.make_params(**_params(model, 3)), seed=9)
+    eng.begin(64, 0.01, 40, 200)
+    eng.advance(33)
+    blob = bytearray(eng.checkpoint())
+    eng.close()
+    header, stride = 224, 64
+    far = np.frombuffer(blob, dtype=np.float32, offset=header + 16 * stride, count=2 * stride).copy()
+    far[3], far[stride + 7] = 3.0e8, -2.5e9
+    blob[header + 16 * stride:header + 24 * stride] = far.tobytes()
+    h = 0xcbf29ce484222325
+    for byte in blob[header:]:
+        h = ((h ^ byte) * 0x100000001b3) & 0xFFFFFFFFFFFFFFFF
+    blob[216:224] = h.to_bytes(8, "little")
+    r = []
+    for grid in (0, 3):
+        eng = E.Engine(model, E.make_params(**_params(model, 3)), seed=9)
+        eng.set_tuning(64, grid)
+        eng.restore(bytes(blob))
+        out = _outputs(64)
+        eng.advance(0, path_out=out)
+        r.append([eng.stats()["sums"]] + [v.cpu().numpy() for v in out.values()])
+        eng.close()
+    for a, b in zip(*r):
+        np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("model", [0, 1, 2])
 @pytest.mark.parametrize("flags", FLAGS)
 def test_split_probes_equal_persistent_probes(E, model, flags):
     """Step-size probes (local_error) of few paths against the one-warp kernel."""
