@@ -402,8 +402,9 @@ __device__ __forceinline__ float three_point(uint32_t& r, const PointConsts& P)
 //  - the drive of a chunk's steps as pairs (d, d), two steps a load, instead
 //    of a shuffle and a move per step.
 // Measured (2^20 dichotomous paths x 20,000 steps): 27.6 warp-instructions per
-// path-step instead of 30.1, 23.1 ms instead of 24.8; the FMA pipe's heavy half
-// (packed pairs and wide multiplies) is then 72 % busy, the SFU 58 %.
+// path-step instead of 30.1, 23.1 ms instead of 24.8 (21.4 with one copy of the
+// step loop, simulate_paths); the FMA pipe's heavy half (packed pairs and wide
+// multiplies) is then 72 % busy, the SFU 60 %.
 constexpr uint32_t kDigitPairs = 36u;
 
 // By all 32 lanes, before the first chunk of a point.
@@ -1320,15 +1321,39 @@ __device__ __forceinline__ void simulate_paths(const PointConsts& P, const Launc
     }
 #pragma unroll
     for (int p = 0; p < PPT; ++p) init_path<MODEL, POIS, DICH>(S[p], P, K, path[p]);
-    run_steps_multi<MODEL, POIS, DICH, GAUSS, false, PPT>(S, P, K, path, lane, 0u, P.n_tr, aux, win);
+    if constexpr (PackedPairs<MODEL, GAUSS, PPT>::value) {
+        // One copy of the step loop for the transient and the averaging window
+        // (the transient's sums are dropped): the warps of an SM soon stand in
+        // different items, and two copies, 14 KB each, run side by side did not
+        // fit the instruction cache.  Measured (2^20 paths x 110,016 steps, one
+        // copy against a transient loop without sums): 1/11 transient 116.3
+        // against 123.2 ms, half 116.3 against 131.2, Poisson noise 132.0 against
+        // 136.2 and 156.1; all but 64 steps transient 116.3 against 111.1.
+#pragma unroll 1
+        for (uint32_t window = 0u; window < 2u; ++window) {
+            run_steps_multi<MODEL, POIS, DICH, GAUSS, true, PPT>(S, P, K, path, lane, window ? P.n_tr : 0u,
+                                                                 P.n_tr + (window ? P.n_avg : 0u), aux, win);
+            if (window) break;
 #pragma unroll
-    for (int p = 0; p < PPT; ++p) {
-        if (!FoldPerStep<MODEL>::value) fold<MODEL>(S[p]);
-        S[p].c_i = S[p].c;
-        S[p].kf_i = S[p].kf;
+            for (int p = 0; p < PPT; ++p) {
+                fold<MODEL>(S[p]);
+                S[p].c_i = S[p].c;
+                S[p].kf_i = S[p].kf;
+                S[p].svd = S[p].sv2d = 0.0;
+                S[p].sv = S[p].sv2 = 0.0f;
+            }
+        }
+    } else {
+        run_steps_multi<MODEL, POIS, DICH, GAUSS, false, PPT>(S, P, K, path, lane, 0u, P.n_tr, aux, win);
+#pragma unroll
+        for (int p = 0; p < PPT; ++p) {
+            if (!FoldPerStep<MODEL>::value) fold<MODEL>(S[p]);
+            S[p].c_i = S[p].c;
+            S[p].kf_i = S[p].kf;
+        }
+        run_steps_multi<MODEL, POIS, DICH, GAUSS, MODEL == kModelInertial, PPT>(S, P, K, path, lane, P.n_tr,
+                                                                                P.n_tr + P.n_avg, aux, win);
     }
-    run_steps_multi<MODEL, POIS, DICH, GAUSS, MODEL == kModelInertial, PPT>(S, P, K, path, lane, P.n_tr,
-                                                                            P.n_tr + P.n_avg, aux, win);
 #pragma unroll
     for (int p = 0; p < PPT; ++p) finish_path<MODEL, POIS, DICH>(S[p], P, R[p]);
 }
