@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(128, 6) scan_kernel(const PointConsts* __restr
         const uint32_t path = it.y + lane;
         const bool valid = path < P.n_paths;
         PathResult R;
-        simulate_path<kModelInertial, POIS, DICH, GAUSS, kKickWin>(P, K, path, lane, R, win);
+        simulate_path<kModelInertial, POIS, DICH, GAUSS, kKickWin, true>(P, K, path, lane, R, win);
         store_partial(partials, item, lane, valid, R);
     }
 }
