@@ -49,7 +49,10 @@ int sde_mlp_set_maps(sde_mlp* net, const float* shift, const float* scale, uint3
                      const float* out_shift, const float* out_scale);
 
 /* Copy the FP32 master parameters from / to the host (SDE_MLP_NPARAMS floats).
- * Setting them also refreshes the BF16 copies and zeroes the Adam state. */
+ * Setting them also refreshes the BF16 copies, zeroes the Adam state and
+ * clears a training failure.  SDE_ETIMEDOUT from sde_mlp_get_params: a
+ * training step gave up (sde_mlp_set_wait_polls); the parameters copied are
+ * those before it. */
 int sde_mlp_set_params(sde_mlp* net, const float* host_params);
 int sde_mlp_get_params(sde_mlp* net, float* host_params);
 
@@ -99,8 +102,16 @@ int sde_mlp_fit(sde_mlp* net, const float* X, const float* T, uint64_t N, uint64
 int sde_mlp_set_tensor_path(sde_mlp* net, int use_tcgen05);
 
 /* Wait for the network's stream and report device-side failures: SDE_ETIMEDOUT
- * if a tensor-core completion wait ran out of its iteration limit. */
+ * if a tensor-core completion wait ran out of its iteration limit, or a
+ * training step gave up. */
 int sde_mlp_sync(sde_mlp* net);
+
+/* Polls after which a training step gives up waiting for its weights (default
+ * 2^24; 0 gives up at once).  A step that gives up changes no parameter and no
+ * Adam moment, nor does any step after it until sde_mlp_set_params;
+ * sde_mlp_fit, sde_mlp_gradients, sde_mlp_get_params and sde_mlp_sync then
+ * return SDE_ETIMEDOUT (sde_mlp_train_step does not wait for its result). */
+int sde_mlp_set_wait_polls(sde_mlp* net, uint32_t polls);
 
 /* Building block exposed for tests: C[M][N] (FP32, device) = op(A) op(B) with
  * BF16 operands on the tensor cores.  a_layout 0: A is [M][K] row-major,

@@ -319,7 +319,7 @@ struct sde_mlp {
     uint64_t h2_rows = 0;
     CUtensorMap h2_store{}, h2_load{};
     int sm_count = 0;
-    int* tc_error = nullptr;         // device word set by a timed-out tensor-core wait
+    int* tc_error = nullptr;         // device words set when a wait ran out: [0] forward, [1] training
 };
 
 static std::string g_mlp_error;
@@ -430,6 +430,14 @@ static sde_train::Update adam_update(float lr, float beta1, float beta2, float e
     return u;
 }
 
+// After a synchronisation: whether a training step gave up.
+static int train_status(sde_mlp* n)
+{
+    if (*n->train.report == 0) return SDE_OK;
+    return mfail(n, SDE_ETIMEDOUT, "a training step's wait for its weights ran out; the parameters are those before that "
+                                   "step and stay so until sde_mlp_set_params");
+}
+
 extern "C" {
 
 const char* sde_mlp_last_error(const sde_mlp* n) { return n ? n->err.c_str() : g_mlp_error.c_str(); }
@@ -457,19 +465,21 @@ int sde_mlp_create(sde_mlp** out, uint64_t seed, void* cuda_stream)
     if (e == cudaSuccess) e = cudaMalloc(&n->m2, P * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&n->maps, 32 * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&n->loss64, sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&n->tc_error, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(n->tc_error, 0, sizeof(int));
+    if (e == cudaSuccess) e = cudaMalloc(&n->tc_error, 2 * sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(n->tc_error, 0, 2 * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&n->train.loss_part, sde_train::kLossBlocks * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&n->train.loss_done, sizeof(uint32_t));
     if (e == cudaSuccess) e = cudaMemset(n->train.loss_done, 0, sizeof(uint32_t));
     if (e == cudaSuccess) e = sde_train::weight_maps(n->wb, &n->train.w2, &n->train.w3);
-    n->train.error = n->tc_error;
+    n->train.error = n->tc_error + 1;
+    n->train.polls = sde_train::kDefaultPolls;
     if (e == cudaSuccess) {
         int dev = 0;
         e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n->sm_count, cudaDevAttrMultiProcessorCount, dev);
     }
     if (e == cudaSuccess) e = cudaMallocHost(&n->host_loss, sizeof(double));
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&n->train.report, sizeof(int));
     if (e != cudaSuccess) {
         mfail(nullptr, SDE_ECUDA, std::string("sde_mlp_create: ") + cudaGetErrorString(e));
         sde_mlp_destroy(n);
@@ -539,7 +549,9 @@ int sde_mlp_set_params(sde_mlp* n, const float* host)
     MLP_CUDA(n, cudaGetLastError());
     MLP_CUDA(n, cudaMemsetAsync(n->m1, 0, P * sizeof(float), n->stream));
     MLP_CUDA(n, cudaMemsetAsync(n->m2, 0, P * sizeof(float), n->stream));
+    MLP_CUDA(n, cudaMemsetAsync(n->train.error, 0, sizeof(int), n->stream));
     MLP_CUDA(n, cudaStreamSynchronize(n->stream));
+    *n->train.report = 0;
     n->step = 0;
     return SDE_OK;
 }
@@ -549,7 +561,7 @@ int sde_mlp_get_params(sde_mlp* n, float* host)
     if (!n || !host) return SDE_EINVAL;
     MLP_CUDA(n, cudaMemcpyAsync(host, n->w, kNParams * sizeof(float), cudaMemcpyDeviceToHost, n->stream));
     MLP_CUDA(n, cudaStreamSynchronize(n->stream));
-    return SDE_OK;
+    return train_status(n);
 }
 
 int sde_mlp_forward(sde_mlp* n, const float* x, uint64_t M, float* y)
@@ -596,6 +608,7 @@ int sde_mlp_gradients(sde_mlp* n, const float* x, const float* t, uint64_t M, fl
     MLP_CUDA(n, cudaMemcpyAsync(host_grad, n->grad, kNParams * sizeof(float), cudaMemcpyDeviceToHost, n->stream));
     MLP_CUDA(n, cudaMemcpyAsync(n->host_loss, n->loss64, sizeof(double), cudaMemcpyDeviceToHost, n->stream));
     MLP_CUDA(n, cudaStreamSynchronize(n->stream));
+    if ((rc = train_status(n))) return rc;
     if (host_loss) *host_loss = *n->host_loss;
     return SDE_OK;
 }
@@ -653,6 +666,7 @@ int sde_mlp_fit(sde_mlp* n, const float* X, const float* T, uint64_t N, uint64_t
     const cudaError_t es = cudaStreamSynchronize(n->fit_stream);
     if (e == cudaSuccess) e = es;
     MLP_CUDA(n, e);
+    if ((rc = train_status(n))) return rc;
     n->step += steps;
     return SDE_OK;
 }
@@ -694,6 +708,13 @@ int sde_mlp_sync(sde_mlp* n)
     int err = 0;
     MLP_CUDA(n, cudaMemcpy(&err, n->tc_error, sizeof(int), cudaMemcpyDeviceToHost));
     if (err) return mfail(n, SDE_ETIMEDOUT, "a tensor-core completion wait ran out (mbarrier not signalled)");
+    return train_status(n);
+}
+
+int sde_mlp_set_wait_polls(sde_mlp* n, uint32_t polls)
+{
+    if (!n) return SDE_EINVAL;
+    n->train.polls = polls;
     return SDE_OK;
 }
 
@@ -719,6 +740,7 @@ void sde_mlp_destroy(sde_mlp* n)
     cudaFree(n->maps); cudaFree(n->loss64); cudaFree(n->tc_error);
     cudaFree(n->train.loss_part); cudaFree(n->train.loss_done);
     if (n->host_loss) cudaFreeHost(n->host_loss);
+    if (n->train.report) cudaFreeHost((void*)n->train.report);
     if (n->fit_stream) cudaStreamDestroy(n->fit_stream);
     if (n->fit_ev) cudaEventDestroy(n->fit_ev);
     if (n->own_stream) cudaStreamDestroy(n->stream);

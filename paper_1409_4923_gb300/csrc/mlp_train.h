@@ -30,6 +30,8 @@ struct Batch {
     uint32_t settled;            // x, t and the maps were complete before the kernel before this step's began
 };
 
+constexpr uint32_t kDefaultPolls = 1u << 24;
+
 // Loss sums: blocks of 256 rows, at most 65536 rows.
 constexpr int kLossBlocks = 256;
 
@@ -50,7 +52,9 @@ struct Net {
     float* res;                  // [cap][2] residuals y' - t'
     double* loss_part;           // [kLossBlocks] partial losses
     uint32_t* loss_done;         // blocks that have written theirs (0 between steps)
-    int* error;                  // set when a wait for a copy ran out
+    int* error;                  // set when a wait for a copy ran out: no later step changes the parameters
+    volatile int* report;        // the same in pinned host memory, for the host to read without a copy
+    uint32_t polls;              // of a wait for a copy, before it gives up
 };
 
 // What to do with the gradients: write them (grad != NULL) or take one Adam

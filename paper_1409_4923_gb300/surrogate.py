@@ -40,6 +40,7 @@ def _lib():
                                                 f, f, P, P]),
             "sde_mlp_set_tensor_path": (ctypes.c_int, [P, ctypes.c_int]),
             "sde_mlp_sync": (ctypes.c_int, [P]),
+            "sde_mlp_set_wait_polls": (ctypes.c_int, [P, ctypes.c_uint32]),
             "sde_mlp_destroy": (None, [P]),
             "sde_mlp_last_error": (ctypes.c_char_p, [P]),
         }
@@ -91,8 +92,12 @@ class Surrogate:
         self._check(self._L.sde_mlp_set_tensor_path(self._net, int(use_tcgen05)))
 
     def sync(self):
-        """Wait for the stream; raises if a tensor-core wait ran out."""
+        """Wait for the stream; raises if a tensor-core wait ran out or a training step gave up."""
         self._check(self._L.sde_mlp_sync(self._net))
+
+    def set_wait_polls(self, polls):
+        """Polls after which a training step gives up waiting for its weights (default 2^24)."""
+        self._check(self._L.sde_mlp_set_wait_polls(self._net, int(polls)))
 
     def get_params(self):
         out = np.zeros(NPARAMS, dtype=np.float32)
