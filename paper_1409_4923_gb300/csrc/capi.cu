@@ -464,20 +464,25 @@ int sde_occupancy(sde_ctx* c, int block_threads, int* blocks_per_sm, int* sm_cou
 
 // Whether coordinates stay below 2^20 between two folds, so that the folds may
 // round by adding 1.5 2^23 (fold<MODEL, true>).  Each step's terms are bounded
-// by the constants: the Gaussian increment by 6 xi (Box-Muller: sqrt(48 ln 2)),
-// a kick by 24 ln 2 zeta; for damping gamma dt <= 1/2 the velocity stays below
-// its initial value plus 8 / (gamma dt) times their sum.  c0, v0: the largest
-// coordinate and velocity of states that come from a checkpoint.
+// by the constants (`step`): the Gaussian increment by 6 xi (Box-Muller:
+// sqrt(48 ln 2)), a kick by 24 ln 2 zeta.  The first fold of a washboard's
+// initial coordinate c leaves half a period and the rounding of c / 2 pi and
+// of the constants, below 2^-22 |c| (the piecewise-linear fold is exact).
+// For damping gamma dt <= 1/2 the velocity stays below its initial value plus
+// 8 / (gamma dt) times `step`.  c0, v0: the largest coordinate and velocity of
+// states that come from a checkpoint.
 static bool near_folds(sde_model model, const PointConsts& P, double c0 = 0.0, double v0 = 0.0)
 {
     const double step = std::fabs((double)P.fdt) + std::fabs((double)P.a_dt) + std::fabs((double)P.F_dt) +
                         6.0 * std::fabs((double)P.xi_c) + 24.0 * std::fabs((double)P.zeta_l2) +
                         std::fabs((double)P.aP_dt) + std::fabs((double)P.Fb_dt) + std::fabs((double)P.mFa_dt);
-    double reach = 4.0 + c0 + 4.0 * step;
+    const double x0 = std::fabs((double)P.x0_lo) + std::fabs((double)P.x0_span);
+    const double first = 4.0 + (model == SDE_OVERDAMPED_PWL ? 0.0 * x0 : std::ldexp(kTwoPi * x0, -21));
+    double reach = first + c0 + 4.0 * step;
     if (model == SDE_INERTIAL_WASHBOARD) {
         if (!(P.gdt > 0.0f && P.gdt <= 0.5f)) return false;
         const double v = v0 + std::fabs((double)P.v0_lo) + std::fabs((double)P.v0_span) + 8.0 * step / (double)P.gdt;
-        reach = 4.0 + c0 + 4.0 * (double)P.wdt * (v + 4.0 * step);
+        reach = first + c0 + 4.0 * (double)P.wdt * (v + 4.0 * step);
     }
     return reach < 1048576.0;      // false for NaN
 }
