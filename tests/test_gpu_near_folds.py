@@ -66,3 +66,29 @@ def test_far_initial_coordinates(E, model, x0):
         assert np.any(near[0] != near[1])
     prm = E.make_params(**dict(_params(model, 3), x0_lo=min(x0, 2 * x0), x0_hi=max(x0, 2 * x0)))
     _same(E, model, prm, lambda eng, out: eng.run(64, 0.01, 40, 200, path_out=out))
+
+
+@pytest.mark.parametrize("model", [0, 1, 2])
+def test_far_coordinates_of_a_checkpoint_where_the_roundings_differ(E, model):
+    """A checkpoint (its checksum valid) whose coordinates the two roundings fold differently."""
+    eng = E.Engine(model, E.make_params(**_params(model, 3)), seed=9)
+    eng.begin(64, 0.01, 40, 200)
+    eng.advance(33)
+    blob = bytearray(eng.checkpoint())
+    eng.close()
+    odd = 2.0 * np.arange(2300000, 2300064) + 1.0             # whole periods, between 2^22 and 2^23
+    c = ((odd * float(TWO_PI)) if model != 2 else 2.0 * odd - 0.5).astype(F32) * np.where(np.arange(64) % 2, 1, -1)
+    c = c.astype(F32)
+    near = _roundings(model, c)
+    assert np.mean(near[0] != near[1]) > 0.25
+    header, stride = 224, 64
+    blob[header + 16 * stride:header + 20 * stride] = c.tobytes()
+    h = 0xcbf29ce484222325
+    for byte in blob[header:]:
+        h = ((h ^ byte) * 0x100000001b3) & 0xFFFFFFFFFFFFFFFF
+    blob[216:224] = h.to_bytes(8, "little")
+
+    def run(eng, out):
+        eng.restore(bytes(blob))
+        eng.advance(0, path_out=out)
+    _same(E, model, E.make_params(**_params(model, 3)), run)
