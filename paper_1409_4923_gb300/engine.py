@@ -74,8 +74,8 @@ def _scan_array(points):
     parts = []
     for pt in points:
         p = pt["params"]
-        if not isinstance(p, Params):
-            raise TypeError("params must be engine.Params")
+        if type(p) is not Params:
+            p = ScanPoint(p).p      # a tuple of field values, or a subclass's part, as ctypes converts it
         parts.append(bytes(p))
         parts.append(_POINT_TAIL.pack(float(pt["dt"]), int(pt["paths"]) & _U64, int(pt["n_transient"]) & _U64,
                                       int(pt["n_avg"]) & _U64))
