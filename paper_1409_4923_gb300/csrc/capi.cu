@@ -468,9 +468,12 @@ int sde_occupancy(sde_ctx* c, int block_threads, int* blocks_per_sm, int* sm_cou
 // sqrt(48 ln 2)), a kick by 24 ln 2 zeta.  The first fold of a washboard's
 // initial coordinate c leaves half a period and the rounding of c / 2 pi and
 // of the constants, below 2^-22 |c| (the piecewise-linear fold is exact).
-// For damping gamma dt <= 1/2 the velocity stays below its initial value plus
-// 8 / (gamma dt) times `step`.  c0, v0: the largest coordinate and velocity of
-// states that come from a checkpoint.
+// With g = gamma dt <= 2 no stage of a step enlarges the velocity; a step
+// multiplies it by rho = |1 - g + g^2/2 - g^3/4| and adds up to 1 + g/2 + g^2/4
+// times `step`, so that it stays below its initial value plus a geometric sum
+// of those (below 8 / g for g <= 1/2; 2^-21: the rounding of a step's
+// operations).  c0, v0: the largest coordinate and velocity of states that
+// come from a checkpoint.
 static bool near_folds(sde_model model, const PointConsts& P, double c0 = 0.0, double v0 = 0.0)
 {
     const double step = std::fabs((double)P.fdt) + std::fabs((double)P.a_dt) + std::fabs((double)P.F_dt) +
@@ -480,18 +483,26 @@ static bool near_folds(sde_model model, const PointConsts& P, double c0 = 0.0, d
     const double first = 4.0 + (model == SDE_OVERDAMPED_PWL ? 0.0 * x0 : std::ldexp(kTwoPi * x0, -21));
     double reach = first + c0 + 4.0 * step;
     if (model == SDE_INERTIAL_WASHBOARD) {
-        if (!(P.gdt > 0.0f && P.gdt <= 0.5f)) return false;
-        const double v = v0 + std::fabs((double)P.v0_lo) + std::fabs((double)P.v0_span) + 8.0 * step / (double)P.gdt;
+        const double g = (double)P.gdt;
+        if (!(g > 0.0 && g <= 2.0)) return false;
+        double grown = 1.0, sum = 8.0 / g;
+        if (g > 0.5) {
+            const double rho = std::fabs(1.0 - g + 0.5 * g * g - 0.25 * g * g * g) + std::ldexp(1.0, -21);
+            grown = std::max(1.0, std::pow(rho, (double)P.n_tr + (double)P.n_avg));
+            sum = 3.0 * (rho < 1.0 ? 1.0 / (1.0 - rho) : grown * ((double)P.n_tr + (double)P.n_avg));
+        }
+        const double v = grown * (v0 + std::fabs((double)P.v0_lo) + std::fabs((double)P.v0_span)) + step * sum;
         reach = first + c0 + 4.0 * (double)P.wdt * (v + 4.0 * step);
     }
     return reach < 1048576.0;      // false for NaN
 }
 
-// Paths per lane of a run: the packed pairs of the inertial model fold as
-// near_folds allows, others keep one path per lane (the results are the same).
-static int lane_paths(const sde_ctx* c, bool near)
+// Paths per lane of a point: the packed pairs of the inertial model fold as
+// near_folds allows, others take one path per lane (the results are the same).
+static int lane_paths(sde_model model, int gauss, const PointConsts& P, int ppt)
 {
-    return c->model == SDE_INERTIAL_WASHBOARD && !near ? 1 : c->paths_per_thread;
+    const bool packed = model == SDE_INERTIAL_WASHBOARD && gauss != kGaussNormal;
+    return ppt == 2 && packed && !near_folds(model, P) ? 1 : ppt;
 }
 
 // Runs of few paths draw their noise in warps of their own (split_kernels.cuh),
@@ -547,7 +558,8 @@ static int run_impl(sde_ctx* c, uint64_t first_path, uint64_t paths, double dt, 
                                      StatePlanes{nullptr, 0u}, 0u, (uint32_t)total, ws, po, c->stream));
         else
             SDE_CUDA(c, launch_point((int)c->model, (f & SDE_NOISE_POISSON) != 0, dich_kind(f),
-                                 gauss_kind(c->p), lane_paths(c, near_folds(c->model, P)), P, K, ws, po, c->block_threads,
+                                 gauss_kind(c->p), lane_paths(c->model, gauss_kind(c->p), P, c->paths_per_thread), P, K, ws, po,
+                                 c->block_threads,
                                  c->grid_blocks, c->sm_count, c->stream));
     } else {
         // Algorithm 5 with `samples` = steps_per_launch: the path states stay
@@ -649,11 +661,12 @@ static int launch_points_fanout(sde_ctx* c, const std::vector<uint32_t>& order,
     for (int k = 0; k < nfan; ++k) SDE_CUDA(c, cudaStreamWaitEvent(c->fan[k], c->fan_ev[kFanStreams], 0));
     for (size_t k = 0; k < order.size(); ++k) {
         const uint32_t i = order[k];
+        const int lanes = lane_paths(c->model, gauss[i], P[i], ppt);
         const LaunchConsts K = make_launch(c->seed, ranges[i].y, budget);
         Workspace wsi{d_counters + i, ws.status, ws.partials + 5ull * ranges[i].x};
         PathOutPtrs po{nullptr, nullptr, nullptr, nullptr, nullptr};
         SDE_CUDA(c, launch_point((int)c->model, (flags & SDE_NOISE_POISSON) != 0, dich_kind(flags), gauss[i],
-                                 ppt, P[i], K, wsi, po, c->block_threads, c->grid_blocks, c->sm_count,
+                                 lanes, P[i], K, wsi, po, c->block_threads, c->grid_blocks, c->sm_count,
                                  c->fan[k % nfan]));
     }
     for (int k = 0; k < nfan; ++k) {
@@ -706,20 +719,21 @@ static int scan_impl(sde_ctx* c, const sde_scan_point* pts, uint32_t npts, sde_s
         inertial_scan && (c->scan_mode == 1 ||
                           (c->scan_mode == 0 && (budget > 0 || sum_paths < kPointScanMinPaths * npts)));
     // Per-point launches of the inertial model take two paths per lane where
-    // the packed pairs apply (near_folds for every point), with Poisson noise
+    // the packed pairs apply (near_folds of the point), with Poisson noise
     // too (measured on the 64 x 64 Poisson scan: 3.75 s against 3.81 s with one
-    // path per lane).  Without Poisson noise the scan kernel does as well: a
-    // work item is 64 paths of one point and writes the partial records of its
-    // two 32-path tiles, so each point's records start at an even index (a point
-    // with an odd tile count leaves one record unused and unfolded).
+    // path per lane).  Without Poisson noise the scan kernel does as well, if
+    // they apply to every point: a work item is 64 paths of one point and
+    // writes the partial records of its two 32-path tiles, so each point's
+    // records start at an even index (a point with an odd tile count leaves one
+    // record unused and unfolded).
     bool near = true;
     for (uint32_t i = 0; i < npts; ++i) {
         int rc = make_point(c, c->model, pts[i].p, pts[i].dt, pts[i].paths, pts[i].n_transient,
                             pts[i].n_avg, P[i]);
         if (rc) return rc;
-        near = near && near_folds(c->model, P[i]);
+        near = near && (!use_scan_kernel || near_folds(c->model, P[i]));
     }
-    const int point_ppt = inertial_scan ? (near ? 2 : 1) : lane_paths(c, near);
+    const int point_ppt = inertial_scan ? 2 : c->paths_per_thread;
     const bool x2 = use_scan_kernel && near && !(flags & SDE_NOISE_POISSON);
     const uint64_t item_paths = x2 ? 64ull : 32ull;
     std::vector<uint2> ranges(npts), items;

@@ -92,3 +92,23 @@ def test_far_coordinates_of_a_checkpoint_where_the_roundings_differ(E, model):
         eng.restore(bytes(blob))
         eng.advance(0, path_out=out)
     _same(E, model, E.make_params(**_params(model, 3)), run)
+
+
+@pytest.mark.parametrize("dt", [0.6, 0.9, 1.6, 2.2, 2.5])
+def test_strong_damping_per_step(E, dt):
+    """gamma dt from 0.54 to 2.25, up to and past the stability limit of a step
+    (where paths may run off to infinities): packed pairs and few-path kernels
+    against the persistent kernel, in runs and in a scan whose other points are
+    ordinary ones or far beyond the near folds' range."""
+    prm = E.make_params(**_params(0, 3))
+    _same(E, 0, prm, lambda eng, out: eng.run(64, dt, 40, 200, path_out=out))
+    points = [dict(params=p, dt=d, paths=100, n_transient=10, n_avg=200)
+              for p, d in ((prm, dt), (prm, 0.01), (E.make_params(**dict(_params(0, 3), zeta=1e9)), 0.01), (prm, dt))]
+    sums = []
+    for mode in (1, 2):
+        eng = E.Engine(0, prm, seed=9)
+        eng.set_tuning(64, 3)
+        eng.set_scan_mode(mode)
+        sums.append([r["sums"] for r in eng.scan(points)])
+        eng.close()
+    np.testing.assert_array_equal(sums[0], sums[1])
