@@ -282,13 +282,20 @@ int sde_philox_words(sde_ctx* ctx, const uint32_t* ctr, uint64_t n, uint64_t see
 /* Launch shape of the path kernels of this context: threads per block
  * (32..128, multiple of 32) and blocks in the grid (0 = one persistent wave
  * from the occupancy calculator).  Without a grid, runs, segments and step-size
- * probes of few paths (up to eight 32-path blocks per SM, 24 with Box-Muller
- * increments) take kernels whose noise is drawn by warps of their own, and the
- * block size does not apply to them.  Results never depend on the shape; the
+ * probes of few paths (six to 24 32-path blocks per SM by noise and model, see
+ * sde_few_paths_limit) take kernels whose noise is drawn by warps of their own,
+ * and the block size does not apply to them.  Results never depend on the shape; the
  * autotuner of the Python layer picks it.  EINVAL outside those ranges.
  * Tuning aid: the paper fixes no launch shape (Sec. 5 only asks for enough
  * threads per block to keep the GPU busy). */
 int sde_set_tuning(sde_ctx* ctx, int block_threads, int grid_blocks);
+
+/* The largest path count for which a run with these parameters, in one launch
+ * and without a grid set by hand, takes the few-path kernels on the current
+ * device (0: never).  For callers that keep launch shapes per path count, as
+ * the autotuner of the Python layer does.  EINVAL for parameters that
+ * sde_create refuses. */
+int sde_few_paths_limit(sde_model model, const sde_params* p, uint64_t* paths);
 
 /* Paths integrated by one GPU lane (1 or 2; default 1).  With 2, each lane
  * advances two paths step by step, interleaved, so that their independent

@@ -505,21 +505,65 @@ static int lane_paths(sde_model model, int gauss, const PointConsts& P, int ppt)
     return ppt == 2 && packed && !near_folds(model, P) ? 1 : ppt;
 }
 
-// Runs of few paths draw their noise in warps of their own (split_kernels.cuh),
-// up to eight 32-path blocks per SM (two integrating warps per scheduler), with
-// Box-Muller up to 24.  Measured (4096 steps, this against one warp per 32 paths
-// with the draws in line, microseconds):
-//   32-path blocks          32          608         1216        1824        3648
-//   Poisson + 3-point    183 / 269   221 / 281   330 / 330   471 / 417   862 / 760
-//   dichotomous + 3-p.   194 / 318   230 / 330   341 / 380   479 / 466   874 / 837
-//   Poisson + Box-M.     218 / 544   292 / 557   454 / 641   686 / 753  1186 / 1331
-//   piecewise-linear P.  281 / 452   296 / 465   391 / 491   590 / 529  1007 / 803
-// A grid set by hand keeps the persistent kernel.
-static bool use_split(const sde_ctx* c, uint64_t items, int dich, int gauss, uint32_t flags, const PointConsts& P,
+// Runs of few paths draw their noise in warps of their own (split_kernels.cuh)
+// up to this many 32-path blocks per SM.  kRun: a whole run in one launch,
+// against the point kernel; kCut: launches that keep the states, against the
+// segment kernel; kProbe: step-size probes, against chi_kernel.  Where the
+// lines lie and why (2048 steps, 152 SMs, this against one warp per 32 paths
+// with the draws in line, microseconds; inertial / overdamped washboard /
+// piecewise-linear where not named):
+//  - eight: two integrating warps per scheduler; one beside the draws is what
+//    the other kernels have.  At eight: three-point alone 205 / 240 piecewise-
+//    linear, Poisson 176 / 195, 175 / 231, 213 / 283, Poisson + three-point
+//    196 / 212, 208 / 241, 223 / 306, dichotomous + three-point 187 / 204, both
+//    jumps + three-point 238 / 273, 229 / 292, 275 / 364.  At twelve (Poisson +
+//    three-point, 4096 steps) 471 / 417;
+//  - six for the inertial model with three-point increments alone, whose other
+//    kernel draws little: at six 136 / 146, at seven 166 / 146 (cut: six
+//    151 / 177, eight 185 / 176);
+//  - six for both jumps with the dichotomous drift and three-point increments,
+//    whose 33 KB of shared memory let no seventh block onto an SM: at six
+//    233 / 274, 229 / 290, 271 / 358, at seven 330 / 275, 360 / 294, 415 / 362
+//    (cut, at eight: 376 / 708, 404 / 719, 464 / 780);
+//  - 24 with Box-Muller increments, drawn by two warps more: at 24
+//    Box-Muller alone 518 / 544, 508 / 521, 589 / 614, with Poisson 647 / 1163,
+//    657 / 1123, 825 / 1236, all three 786 / 1313, 777 / 1253, 982 / 1367;
+//  - fourteen for Box-Muller and dichotomous noise in the overdamped models:
+//    at fourteen 409 / 445 and 495 / 516, at sixteen 460 / 447 and 545 / 519
+//    (cut: 487 / 484 and 559 / 557; inertial at 24: 644 / 657);
+//  - probes: their other kernel draws a Philox block for every step; at eight
+//    33..56 / 60..108, with Box-Muller at 24 62..107 / 113..176.
+enum SplitUse { kRun, kCut, kProbe };
+static uint64_t split_blocks_per_sm(sde_model model, uint32_t flags, int gauss, SplitUse use)
+{
+    const bool pois = (flags & SDE_NOISE_POISSON) != 0, inertial = model == SDE_INERTIAL_WASHBOARD;
+    const int dich = dich_kind(flags);
+    if (!pois && !dich && !gauss) return 0;          // nothing to draw
+    if (gauss == kGaussNormal) return use != kProbe && !inertial && dich && !pois ? 14 : 24;
+    if (use != kProbe && inertial && !pois && !dich) return 6;
+    if (use == kRun && pois && dich == 2 && gauss) return 6;
+    return 8;
+}
+
+// A grid set by hand keeps the other kernels.
+static bool use_split(const sde_ctx* c, uint64_t items, int gauss, uint32_t flags, SplitUse use, const PointConsts& P,
                       double c0 = 0.0, double v0 = 0.0)
 {
-    return c->grid_blocks == 0 && items <= (gauss == kGaussNormal ? 24ull : 8ull) * (uint64_t)c->sm_count &&
-           ((flags & SDE_NOISE_POISSON) || dich || gauss) && near_folds(c->model, P, c0, v0);
+    return c->grid_blocks == 0 && items <= split_blocks_per_sm(c->model, flags, gauss, use) * (uint64_t)c->sm_count &&
+           near_folds(c->model, P, c0, v0);
+}
+
+int sde_few_paths_limit(sde_model model, const sde_params* p, uint64_t* paths)
+{
+    if (!paths) return SDE_EINVAL;
+    int rc = validate_params(nullptr, model, p);
+    if (rc) return rc;
+    int device = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    if (e != cudaSuccess) return cuda_fail(nullptr, e, "sde_few_paths_limit");
+    *paths = 32ull * split_blocks_per_sm(model, p->noise_flags, gauss_kind(*p), kRun) * (uint64_t)sms;
+    return SDE_OK;
 }
 
 static int run_impl(sde_ctx* c, uint64_t first_path, uint64_t paths, double dt, uint64_t n_tr,
@@ -551,8 +595,9 @@ static int run_impl(sde_ctx* c, uint64_t first_path, uint64_t paths, double dt, 
     const LaunchConsts K = make_launch(c->seed, (uint32_t)items, 0);
     const uint32_t f = c->p.noise_flags;
     const uint64_t total = n_tr + n_avg;
-    const bool split = use_split(c, items, dich_kind(f), gauss_kind(c->p), f, P);
-    if (c->steps_per_launch == 0 || c->steps_per_launch >= total) {
+    const bool whole = c->steps_per_launch == 0 || c->steps_per_launch >= total;
+    const bool split = use_split(c, items, gauss_kind(c->p), f, whole ? kRun : kCut, P);
+    if (whole) {
         if (split)
             SDE_CUDA(c, launch_split((int)c->model, (f & SDE_NOISE_POISSON) != 0, dich_kind(f), gauss_kind(c->p), P, K,
                                      StatePlanes{nullptr, 0u}, 0u, (uint32_t)total, ws, po, c->stream));
@@ -987,7 +1032,7 @@ int sde_advance(sde_ctx* c, uint64_t n_steps, const sde_path_out* out, uint64_t*
     const LaunchConsts K = make_launch(r.seed, r.items, 0);
     const StatePlanes M{(unsigned char*)c->state, r.stride};
     const uint32_t f = r.p.noise_flags;
-    if (use_split(c, r.items, dich_kind(f), gauss_kind(r.p), f, P, r.c0, r.v0))
+    if (use_split(c, r.items, gauss_kind(r.p), f, kCut, P, r.c0, r.v0))
         SDE_CUDA(c, launch_split((int)c->model, (f & SDE_NOISE_POISSON) != 0, dich_kind(f), gauss_kind(r.p), P, K, M,
                                  (uint32_t)na, (uint32_t)nb, ws, po, c->stream));
     else
@@ -1132,7 +1177,7 @@ int sde_local_error(sde_ctx* c, uint64_t paths, double dt, uint64_t n_steps, dou
     Workspace ws{(uint32_t*)base, (int32_t*)(base + 4), (double*)(base + L.off_partials)};
     const LaunchConsts K = make_launch(c->seed, (uint32_t)items, 0);
     const uint32_t f = c->p.noise_flags;
-    if (use_split(c, items, dich_kind(f), gauss_kind(c->p), f, P)) {
+    if (use_split(c, items, gauss_kind(c->p), f, kProbe, P)) {
         SDE_CUDA(c, launch_split_chi((int)c->model, (f & SDE_NOISE_POISSON) != 0, dich_kind(f), gauss_kind(c->p), P, K,
                                      (uint32_t)n_steps, ws, c->stream));
     } else {

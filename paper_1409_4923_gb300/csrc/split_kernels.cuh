@@ -354,7 +354,7 @@ cudaError_t launch_split_t(const PointConsts& P, const LaunchConsts& K, const St
                            const Workspace& ws, const PathOutPtrs& po, cudaStream_t st)
 {
     if constexpr (SplitLayout<POIS, DICH, GAUSS>::planes == 0) {
-        return cudaErrorInvalidValue;      // nothing to draw (split_applies)
+        return cudaErrorInvalidValue;      // nothing to draw (split_blocks_per_sm is 0)
     } else {
         split_kernel<MODEL, POIS, DICH, GAUSS><<<K.n_items, SplitWarps<POIS, DICH, GAUSS>::threads, SplitLayout<POIS, DICH, GAUSS>::bytes, st>>>(
             P, K, M, na, nb, ws.partials, po);

@@ -130,6 +130,8 @@ def lib():
         "sde_reduce_f64": (ctypes.c_int, [_P, _P, ctypes.c_uint64, ctypes.POINTER(ctypes.c_double)]),
         "sde_philox_words": (ctypes.c_int, [_P, _P, ctypes.c_uint64, ctypes.c_uint64, _P]),
         "sde_set_tuning": (ctypes.c_int, [_P, ctypes.c_int, ctypes.c_int]),
+        "sde_few_paths_limit": (ctypes.c_int, [ctypes.c_int, ctypes.POINTER(Params),
+                                               ctypes.POINTER(ctypes.c_uint64)]),
         "sde_set_paths_per_thread": (ctypes.c_int, [_P, ctypes.c_int]),
         "sde_set_steps_per_launch": (ctypes.c_int, [_P, ctypes.c_uint64]),
         "sde_set_scan_mode": (ctypes.c_int, [_P, ctypes.c_int]),
@@ -181,6 +183,16 @@ def _stream_handle(stream):
     if isinstance(stream, int):
         return ctypes.c_void_p(stream)
     return ctypes.c_void_p(stream.cuda_stream)
+
+
+def few_paths_limit(model, params: Params) -> int:
+    """sde_few_paths_limit: the largest path count for which a run without a fixed
+    grid takes the few-path kernels on the current device."""
+    limit = ctypes.c_uint64()
+    rc = lib().sde_few_paths_limit(int(model), ctypes.byref(params), ctypes.byref(limit))
+    if rc != SDE_OK:
+        raise SdeError(rc, lib().sde_last_error(None).decode())
+    return limit.value
 
 
 class Engine:
