@@ -54,8 +54,17 @@ def size_class(paths):
     return int(math.log(max(paths, 1), 4))
 
 
-def key(device_name, model, flags, paths):
-    return "%s|model=%d|flags=%d|paths~4^%d" % (device_name, model, flags, size_class(paths))
+# Entries of runs tuned with kernels of another generation are not used: a
+# fixed grid that was best before the runs of few paths had kernels of their
+# own keeps them from those kernels (1024 Poisson paths: 1.5 times slower).
+KERNEL_GENERATION = 2
+
+
+def key(device_name, model, flags, paths, few=False):
+    """Cache key of a run's shape.  A size class can span the few-path limit, so
+    the side of it that the run is on belongs to the key."""
+    return "%s|gen=%d|model=%d|flags=%d|paths~4^%d%s" % (device_name, KERNEL_GENERATION, model, flags,
+                                                         size_class(paths), "|few" if few else "")
 
 
 def candidates(sm_count):
@@ -92,11 +101,14 @@ def tune(model, params, dt, paths, n_probe_steps=2048, seed=0, stream=None, cach
     """Time every candidate on a probe of `paths` paths x n_probe_steps steps
     (shape stage), then the steps-per-launch candidates on 2 x n_probe_steps
     steps with the best shape; caches and returns a dict with keys block,
-    grid, ppt, steps_per_launch (and seconds, the probe timings, when it ran)."""
+    grid, ppt, steps_per_launch (and seconds, the probe timings, when it ran).
+    Runs of few paths have one candidate, the default: without a grid all shapes
+    run the same few-path kernel, and a grid would keep them from it."""
     import torch
     cache = cache or cache_path()
     dev = torch.cuda.get_device_name(torch.cuda.current_device())
-    k = key(dev, model, params.noise_flags, paths)
+    few = paths <= E.few_paths_limit(model, params)
+    k = key(dev, model, params.noise_flags, paths, few)
     data = _load(cache)
     if not force and k in data and all(f in data[k] for f in DEFAULT):
         return {f: data[k][f] for f in DEFAULT}
@@ -106,7 +118,7 @@ def tune(model, params, dt, paths, n_probe_steps=2048, seed=0, stream=None, cach
         eng.run(paths, dt, 0, n_probe_steps)         # warm-up (module load, workspace)
         eng.stats()
         shapes = {}
-        for b, g, ppt in candidates(sms):
+        for b, g, ppt in candidates(sms)[:1 if few else None]:
             eng.set_paths_per_thread(ppt)
             eng.set_tuning(b, g)
             shapes[(b, g, ppt)] = _time_run(eng, paths, dt, n_probe_steps)
