@@ -21,6 +21,7 @@
 #include "sde_mlp.h"
 #include "mlp_train.h"
 
+cudaError_t sde_tc_prepare();
 cudaError_t sde_tc_h2_maps(__nv_bfloat16* h2, uint64_t rows, CUtensorMap* store, CUtensorMap* load);
 cudaError_t sde_tc_forward(int M, const float* x, const float* maps, uint32_t log_mask,
                            const __nv_bfloat16* W1, const float* b1, const CUtensorMap& w2, const float* b2,
@@ -470,6 +471,8 @@ int sde_mlp_create(sde_mlp** out, uint64_t seed, void* cuda_stream)
     if (e == cudaSuccess) e = cudaMalloc(&n->train.loss_part, sde_train::kLossBlocks * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&n->train.loss_done, sizeof(uint32_t));
     if (e == cudaSuccess) e = cudaMemset(n->train.loss_done, 0, sizeof(uint32_t));
+    if (e == cudaSuccess) e = sde_train::prepare();
+    if (e == cudaSuccess) e = sde_tc_prepare();
     if (e == cudaSuccess) e = sde_train::weight_maps(n->wb, &n->train.w2, &n->train.w3);
     n->train.error = n->tc_error + 1;
     n->train.polls = sde_train::kDefaultPolls;

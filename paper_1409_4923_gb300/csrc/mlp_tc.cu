@@ -787,10 +787,6 @@ cudaError_t sde_tc_h2_maps(__nv_bfloat16* h2, uint64_t rows, CUtensorMap* store,
 static cudaError_t launch_layers34(const sde_tc::TcArgs& a, const CUtensorMap& w3, const CUtensorMap& h2_load,
                                    int sm_count, cudaStream_t st)
 {
-    // the attribute belongs to the current device: set it on every launch
-    cudaError_t e = cudaFuncSetAttribute(sde_tc::mlp_tc_layers34_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         sde_tc::kL34SmemBytes);
-    if (e != cudaSuccess) return e;
     const int tiles = (a.M + sde_tc::kRows - 1) / sde_tc::kRows;
     const int grid = tiles < sm_count ? tiles : sm_count;
     // programmatic dependent launch: the kernel waits for the layers 1-2 grid
@@ -811,14 +807,22 @@ static cudaError_t launch_layers34(const sde_tc::TcArgs& a, const CUtensorMap& w
 static cudaError_t launch_layers12(const sde_tc::TcArgs& a, const CUtensorMap& w2, const CUtensorMap& h2_store,
                                    int sm_count, cudaStream_t st)
 {
-    // the attribute belongs to the current device: set it on every launch
-    cudaError_t e = cudaFuncSetAttribute(sde_tc::mlp_tc_layers12_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         sde_tc::kL12SmemBytes);
-    if (e != cudaSuccess) return e;
     const int tiles = (a.M + sde_tc::kRows - 1) / sde_tc::kRows;
     const int grid = tiles < sm_count ? tiles : sm_count;
     sde_tc::mlp_tc_layers12_kernel<<<grid, sde_tc::kL12Threads, sde_tc::kL12SmemBytes, st>>>(a, w2, h2_store);
     return cudaGetLastError();
+}
+
+// The kernels' shared-memory limits on the current device; once per network,
+// which stays on its device.
+cudaError_t sde_tc_prepare()
+{
+    cudaError_t e = cudaFuncSetAttribute(sde_tc::mlp_tc_layers12_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         sde_tc::kL12SmemBytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(sde_tc::mlp_tc_layers34_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 sde_tc::kL34SmemBytes);
+    return e;
 }
 
 // Host launcher (used by mlp.cu): the forward pass of M rows of raw inputs x

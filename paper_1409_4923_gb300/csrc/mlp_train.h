@@ -69,6 +69,11 @@ struct Update {
 // Tensor maps of the BF16 parameter copies wb, for Net.w2 and Net.w3.
 cudaError_t weight_maps(const __nv_bfloat16* wb, CUtensorMap* w2, CUtensorMap* w3);
 
+// The kernels' shared-memory limits on the current device; once per network,
+// which stays on its device (on every launch they were two more runtime calls
+// a step from a host that the steps wait for).
+cudaError_t prepare();
+
 // Loss and gradients of the batch, then the update; two kernels on `st`.
 cudaError_t step(const Net& n, const Batch& b, const Update& u, cudaStream_t st);
 
