@@ -480,6 +480,7 @@ int sde_mlp_create(sde_mlp** out, uint64_t seed, void* cuda_stream)
         int dev = 0;
         e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n->sm_count, cudaDevAttrMultiProcessorCount, dev);
+        n->train.sm_count = (uint32_t)n->sm_count;
     }
     if (e == cudaSuccess) e = cudaMallocHost(&n->host_loss, sizeof(double));
     if (e == cudaSuccess) e = cudaMallocHost((void**)&n->train.report, sizeof(int));

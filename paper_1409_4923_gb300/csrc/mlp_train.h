@@ -55,6 +55,7 @@ struct Net {
     int* error;                  // set when a wait for a copy ran out: no later step changes the parameters
     volatile int* report;        // the same in pinned host memory, for the host to read without a copy
     uint32_t polls;              // of a wait for a copy, before it gives up
+    uint32_t sm_count;
 };
 
 // What to do with the gradients: write them (grad != NULL) or take one Adam
