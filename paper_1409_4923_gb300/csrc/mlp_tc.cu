@@ -501,8 +501,8 @@ __global__ void __launch_bounds__(kL12Threads, 1) mlp_tc_layers12_kernel(const _
                 if (j & 1u) {
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
-                    // the box's first row; rows past M are not written, and a box wholly
-                    // past M is not issued
+                    // the box's first row; a box that crosses M is stored whole (the
+                    // buffer has whole tiles), one wholly past M is not issued
                     const int y0 = row - (int)lane;
                     if (lane == 0 && y0 < g.M) {
                         asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
@@ -530,7 +530,8 @@ __global__ void __launch_bounds__(kL12Threads, 1) mlp_tc_layers12_kernel(const _
 
 // ---------------------------------------------------------------------------
 // Layers 3-4 and the output map.  Warp 16 loads K-block c of each h2 tile by
-// TMA (128-byte swizzle, rows past M zero-filled) into slot c as soon as the
+// TMA (128-byte swizzle; rows past M hold whatever the buffer holds: rows are
+// independent, and their outputs are not written) into slot c as soon as the
 // MMAs of the previous tile that read slot c are complete; warp 17 issues a
 // block's four MMAs as soon as its copy has landed; warps 0-15 drain (warp w:
 // lane quarter w mod 4, column quarter w / 4), form layer 4's partial dot
@@ -764,8 +765,9 @@ static EncodeTiledFn lookup_encode_tiled()
 // kernels: layers 1-2 store 32 x 32 boxes from 64-byte-swizzled staging blocks,
 // layers 3-4 load 128-row x 64-column boxes in the 128-byte-swizzled K-major
 // layout of the tensor core's A operand.  They describe the whole buffer, so
-// they serve every call: rows past the call's M that its last tile covers are
-// stored and loaded like the others, and their outputs are not written.
+// they serve every call: its last tile loads rows past its M as the buffer
+// holds them (the last box's are stored, boxes wholly past M are not), and
+// their outputs are not written.
 cudaError_t sde_tc_h2_maps(__nv_bfloat16* h2, uint64_t rows, CUtensorMap* store, CUtensorMap* load)
 {
     static const EncodeTiledFn encode = lookup_encode_tiled();
