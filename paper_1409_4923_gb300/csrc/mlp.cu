@@ -314,7 +314,7 @@ struct sde_mlp {
     __nv_bfloat16* dH[3] = {nullptr, nullptr, nullptr};        // [cap][256]
     float* res = nullptr;            // [cap][2] residuals
     double* loss64 = nullptr;
-    double* host_loss = nullptr;
+    double* host_loss = nullptr;     // pinned: the FP64 loss, then the training kernels' report word
     int use_tc = 1;                  // forward pass on the fused tcgen05 kernels
     __nv_bfloat16* h2 = nullptr;     // their [h2_rows][256] intermediate, and its tensor maps
     uint64_t h2_rows = 0;
@@ -482,8 +482,8 @@ int sde_mlp_create(sde_mlp** out, uint64_t seed, void* cuda_stream)
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n->sm_count, cudaDevAttrMultiProcessorCount, dev);
         n->train.sm_count = (uint32_t)n->sm_count;
     }
-    if (e == cudaSuccess) e = cudaMallocHost(&n->host_loss, sizeof(double));
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&n->train.report, sizeof(int));
+    if (e == cudaSuccess) e = cudaMallocHost(&n->host_loss, 2 * sizeof(double));
+    n->train.report = (volatile int*)(n->host_loss + 1);
     if (e != cudaSuccess) {
         mfail(nullptr, SDE_ECUDA, std::string("sde_mlp_create: ") + cudaGetErrorString(e));
         sde_mlp_destroy(n);
@@ -744,7 +744,6 @@ void sde_mlp_destroy(sde_mlp* n)
     cudaFree(n->maps); cudaFree(n->loss64); cudaFree(n->tc_error);
     cudaFree(n->train.loss_part); cudaFree(n->train.loss_done);
     if (n->host_loss) cudaFreeHost(n->host_loss);
-    if (n->train.report) cudaFreeHost((void*)n->train.report);
     if (n->fit_stream) cudaStreamDestroy(n->fit_stream);
     if (n->fit_ev) cudaEventDestroy(n->fit_ev);
     if (n->own_stream) cudaStreamDestroy(n->stream);
