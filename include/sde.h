@@ -303,8 +303,9 @@ int sde_few_paths_limit(sde_model model, const sde_params* p, uint64_t* paths);
  * loop work are shared; each path takes exactly the operations it takes with
  * 1, so results do not change.  Applies to sde_run, sde_run_paths and the
  * per-point launches of sde_scan for the overdamped models, and not to runs of
- * few paths (sde_set_tuning) or to parameters whose kicks throw the particle
- * past 2^20 in a step.  EINVAL otherwise.
+ * few paths (sde_few_paths_limit) or, in the inertial model, to parameters that
+ * can put the coordinate 2^20 from its fold (huge kicks or initial positions).
+ * EINVAL otherwise.
  * Tuning aid with no counterpart in the paper, which runs one path per
  * thread (Algorithm 5). */
 int sde_set_paths_per_thread(sde_ctx* ctx, int paths_per_thread);
